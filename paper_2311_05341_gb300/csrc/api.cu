@@ -238,6 +238,11 @@ int launch_range(const dd_plan_s* p, const RangePlan& rp, const void* d_in, int6
                  void* stream, int kind = 0, int64_t x_origin = 0) {
   if (kind > 0) {
     unsigned char* ws = static_cast<unsigned char*>(p->d_ws);
+    if (rp.sums.ok)
+      return launch_forward_sum_rows(p, rp, ws + rp.off_sums,
+                                     reinterpret_cast<int32_t*>(ws + tk::kStatusOffset), d_in,
+                                     stride, d_out, t_begin, t_end, stream, n_out, kind,
+                                     x_origin);
     return launch_forward_pattern(p, rp, ws + rp.off_tile_recs,
                                   reinterpret_cast<int32_t*>(ws + tk::kStatusOffset), d_in,
                                   stride, n_out, d_out, t_begin, t_end, stream, n_out, kind,

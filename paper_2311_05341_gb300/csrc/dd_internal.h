@@ -9,6 +9,7 @@
 
 #include "dd.h"
 #include "fwd_tiled.h"
+#include "sumrows.h"
 
 namespace dd {
 
@@ -59,9 +60,13 @@ struct RangePlan {
   // kind's window alignment, a multiple of the packed kind's); 0 if none.
   int32_t alt_kind = 0;
 
+  // Sum-row tile on the packed copies of integer input (sumrows.h).
+  SumTables sums;
+
   // Byte offsets of the device tables inside the workspace.
   size_t off_shifts = 0;        // int32 [n_dm][n_chan]
   size_t off_tile_recs = 0;     // tk::Rec or tk::PRec [tile_n_blocks][n_chan]
+  size_t off_sums = 0;          // sum-row tables (sums.ok)
   std::vector<unsigned char> tile_recs;  // host image of the records
 };
 
@@ -143,6 +148,13 @@ int launch_forward_pattern(const dd_plan_s* p, const RangePlan& rp, const void* 
                            void* d_out, int64_t t_begin, int64_t t_end, void* stream,
                            int64_t out_stride, int kind = 0, int64_t x_origin = 0,
                            bool widen_slots = true);
+// The sum-row kernel (fwd_sumrows.cu) on packed words of kernel kind `kind`
+// (kU8P, kU16P); d_words, stride, x_origin and the times as
+// launch_forward_pattern.
+int launch_forward_sum_rows(const dd_plan_s* p, const RangePlan& rp, const void* tables,
+                            int32_t* err, const void* d_words, int64_t stride, void* d_out,
+                            int64_t t_begin, int64_t t_end, void* stream, int64_t out_stride,
+                            int kind, int64_t x_origin);
 // Packed uint8 copy for the kU8P tiles (pack.cu): out[c][t] = in[c][t] |
 // in[c][t + pair] << 16 for t in [t_begin, t_end) (0 past n_samp); strides in
 // bytes (in) and 32-bit words (out, a multiple of 4); pair and t_begin

@@ -396,6 +396,19 @@ void choose_tile(RangePlan& rp, int32_t n_chan, dd_dtype dtype) {
     if (try_tile_shape(rp, n_chan, kind, *tk::shape_for(dr))) return;
 }
 
+// choose_tile, then the sum-row tables of a range that may run from a packed
+// copy of integer input at the automatic shape (pair distance 736).
+void choose_kernels(RangePlan& rp, int32_t n_chan, dd_dtype dtype) {
+  choose_tile(rp, n_chan, dtype);
+  rp.sums = SumTables{};
+  const int kind = copy_kind(rp, true);
+  if ((kind != tk::kU8P && kind != tk::kU16P) || rp.shape_request >= 0 ||
+      32 * rp.tile_h != sr::kPairWords)
+    return;
+  const int64_t top = dtype == DD_U16 ? 65535 : dtype == DD_U4 ? 15 : 255;
+  build_sum_tables(rp, n_chan, top * rp.r.bin, tk::packed_pairs(kind), &rp.sums);
+}
+
 // The adjoint of range rp (float32) as a forward transform: with P = s_max,
 // xbar_r[c][u] = sum_d ybar[d][u - s(c, d)] = sum_d Z[d][u + P - s(c, d)] for
 // the cotangent rows Z[d] padded with P zeros on both sides, so it is Eq. 3 on
@@ -443,6 +456,11 @@ void layout_workspace(dd_plan_s* p) {
       rp.off_tile_recs = ws;
       ws += rp.tile_recs.size();
     }
+    if (rp.sums.ok) {
+      ws = align_up(ws, 256);
+      rp.off_sums = ws;
+      ws += rp.sums.bytes.size();
+    }
   };
   for (auto& rp : p->ranges) place(rp);
   for (auto& ar : p->adj) place(ar);
@@ -470,6 +488,8 @@ void layout_workspace(dd_plan_s* p) {
                 rp.shifts.size() * sizeof(int32_t));
     if (rp.tile_ok)
       std::memcpy(p->host_ws.data() + rp.off_tile_recs, rp.tile_recs.data(), rp.tile_recs.size());
+    if (rp.sums.ok)
+      std::memcpy(p->host_ws.data() + rp.off_sums, rp.sums.bytes.data(), rp.sums.bytes.size());
   };
   for (const auto& rp : p->ranges) copy(rp);
   for (const auto& ar : p->adj) copy(ar);
@@ -576,7 +596,7 @@ dd_status build_plan(dd_plan_s* p) {
     }
     rp.adj_span = aspan;
 
-    choose_tile(rp, n_chan, p->dtype);
+    choose_kernels(rp, n_chan, p->dtype);
   }
   p->adj.clear();
   if (p->dtype == DD_F32) {
@@ -593,11 +613,11 @@ bool retile_range(dd_plan_s* p, size_t range, int32_t request, int32_t shape_req
   const int32_t old = rp.tile_request, old_shape = rp.shape_request;
   rp.tile_request = request;
   rp.shape_request = shape_request;
-  choose_tile(rp, p->n_chan, p->dtype);
+  choose_kernels(rp, p->n_chan, p->dtype);
   if ((request > 0 || shape_request >= 0) && !rp.tile_ok) {
     rp.tile_request = old;
     rp.shape_request = old_shape;
-    choose_tile(rp, p->n_chan, p->dtype);
+    choose_kernels(rp, p->n_chan, p->dtype);
     layout_workspace(p);
     return false;
   }

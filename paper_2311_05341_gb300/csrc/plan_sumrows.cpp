@@ -1,0 +1,329 @@
+// plan_sumrows.cpp -- host tables of the sum-row tile (sumrows.h): the channel
+// groups of every block of 128 trial DMs, the distinct shift-difference
+// vectors of each group (its sum rows) and the moves that make one row from
+// the next.
+#include <algorithm>
+#include <atomic>
+#include <cstddef>
+#include <cstring>
+#include <new>
+#include <system_error>
+#include <thread>
+#include <vector>
+
+#include "dd_internal.h"
+#include "sumrows.h"
+
+namespace dd {
+
+namespace {
+
+using namespace sr;
+
+// Shared-memory words per channel and 64 trial DMs x 736 packed words (half of
+// this tile's DMs x twice its words) above which the pattern tile is taken.
+// One word is one lane's 4 bytes of the shared-memory pipe, which bounds both
+// tiles: the pattern tile moves (23 + o_3) words per 4 DMs and 23-word window,
+// about 12000, and gets 3/4 of the pipe, as this tile does.  Measured: 1024
+// channels, 2048 trials (8540 words) 3.85 ms against 5.2 ms.
+constexpr double kMaxWordsPerChannel = 10500.0;
+
+// Difference vectors as bit masks: channel i of the group has kLevels bits,
+// v_i - min of them set, so that the distance of two vectors in samples is
+// the number of differing bits.
+constexpr int kLevels = 4;
+
+struct Mask {
+  uint64_t w[kMaxK * kLevels / 64] = {};
+  int dist(const Mask& o) const {
+    int n = 0;
+    for (size_t i = 0; i < sizeof(w) / 8; ++i) n += __builtin_popcountll(w[i] ^ o.w[i]);
+    return n;
+  }
+};
+
+struct Group {
+  int k = 0;
+  int rows = 0;
+  int rs = 0;
+  int lw = 0;
+};
+
+inline int round_up(int v, int m) { return (v + m - 1) / m * m; }
+
+// Words per channel of a group of k channels with `rows` rows: staging and
+// first row, moves (their number grows a little faster than the rows'), rows
+// written, and the adds' reads.
+double words_per_channel(int k, int rows, int rs) {
+  const double moves = rows * (0.75 + k / 40.0) * (1.0 + 1.0 / kBuild);
+  return ((2.0 * k + moves + rows) * rs + static_cast<double>(kDm) * kWords) / k;
+}
+
+template <typename T>
+void put(std::vector<unsigned char>& v, const T& x) {
+  const size_t n = v.size();
+  v.resize(n + sizeof(T));
+  std::memcpy(v.data() + n, &x, sizeof(T));
+}
+
+// The groups of DM block b: window starts, directory (record offsets from the
+// block's first record) and records.  False where the tile cannot serve it.
+struct Block {
+  std::vector<Dir> dir;
+  std::vector<int32_t> start;
+  std::vector<unsigned char> recs;
+  double words = 0;
+};
+
+bool build_block(const RangePlan& rp, int32_t n_chan, int lane_chans, int64_t b, Block* out) {
+  std::vector<Dir>& dir = out->dir;
+  std::vector<unsigned char>& recs = out->recs;
+  out->start.resize(n_chan);
+  size_t last_head = 0;  // of the latest group, for the flush flag
+  std::vector<int32_t> block(static_cast<size_t>(n_chan) * kDm);  // shifts, DM fastest
+  const int n_real = static_cast<int>(std::min<int64_t>(kDm, rp.n_dm - b * kDm));
+  for (int d = 0; d < n_real; ++d) {
+    const int32_t* row = &rp.shifts[static_cast<size_t>(b * kDm + d) * n_chan];
+    for (int32_t c = 0; c < n_chan; ++c) block[static_cast<size_t>(c) * kDm + d] = row[c];
+  }
+  int32_t c = 0;
+  int since = 0;  // channels in the lanes
+  while (c < n_chan) {
+    const int32_t* s0 = &block[static_cast<size_t>(c) * kDm];
+    const int rs = round_up(kWords + s0[n_real - 1] - s0[0], kBuild);
+    if (s0[n_real - 1] < s0[0] || rs > kRowWords) return false;
+    // Extend the group channel by channel, splitting the DMs into classes
+    // of equal difference vectors, and keep the cheapest size that fits.
+    uint8_t cls[kDm] = {};
+    int n_cls = 1, reach = 0;
+    Group best;
+    double best_cost = 1e30;
+    uint8_t best_cls[kDm];
+    const int kmax = static_cast<int>(std::min<int64_t>({kMaxK, n_chan - c, lane_chans}));
+    for (int k = 1; k <= kmax; ++k) {
+      const int32_t* s = &block[static_cast<size_t>(c + k - 1) * kDm];
+      int lo = s[0] - s0[0], hi = lo;
+      for (int d = 1; d < n_real; ++d) {
+        lo = std::min(lo, s[d] - s0[d]);
+        hi = std::max(hi, s[d] - s0[d]);
+      }
+      if (hi - lo >= kLevels) break;
+      reach = std::max(reach, hi - lo);
+      if (hi > lo) {
+        uint8_t id[kDm * kLevels];
+        std::memset(id, 255, static_cast<size_t>(n_cls) * kLevels);
+        int n = 0;
+        for (int d = 0; d < n_real; ++d) {
+          uint8_t& e = id[cls[d] * kLevels + (s[d] - s0[d] - lo)];
+          if (e == 255) e = static_cast<uint8_t>(n++);
+          cls[d] = e;
+        }
+        n_cls = n;
+      }
+      const int lw = round_up(kAlign - 1 + reach + rs + 1, 4);
+      if (k * lw > kRawWords || n_cls * rs > kRowWords) break;
+      // The first row adds channels in pairs: only the last group may be odd.
+      const double cost = words_per_channel(k, n_cls, rs);
+      if (cost < best_cost && (k % 2 == 0 || c + k == n_chan || kmax == 1)) {
+        best_cost = cost;
+        best.k = k;
+        best.rows = n_cls;
+        best.rs = rs;
+        best.lw = lw;
+        std::memcpy(best_cls, cls, sizeof(best_cls));
+      } else if (cost > 1.25 * best_cost) {
+        break;
+      }
+    }
+    if (best.k == 0) return false;
+
+    // The rows' difference vectors, visited nearest first.
+    std::vector<int32_t> rel_min(best.k);
+    for (int i = 0; i < best.k; ++i) {
+      const int32_t* s = &block[static_cast<size_t>(c + i) * kDm];
+      int lo = s[0] - s0[0];
+      for (int d = 1; d < n_real; ++d) lo = std::min(lo, s[d] - s0[d]);
+      rel_min[i] = lo;
+    }
+    std::vector<Mask> mask(best.rows);
+    std::vector<uint8_t> level(static_cast<size_t>(best.rows) * best.k);
+    std::vector<char> seen(best.rows, 0);
+    for (int d = 0; d < n_real; ++d) {
+      const int r = best_cls[d];
+      if (seen[r]) continue;
+      seen[r] = 1;
+      for (int i = 0; i < best.k; ++i) {
+        const int v = block[static_cast<size_t>(c + i) * kDm + d] - s0[d] - rel_min[i];
+        level[static_cast<size_t>(r) * best.k + i] = static_cast<uint8_t>(v);
+        for (int q = 0; q < v; ++q) {
+          const int bit = i * kLevels + q;
+          mask[r].w[bit / 64] |= uint64_t{1} << (bit % 64);
+        }
+      }
+    }
+    std::vector<int> order;
+    std::vector<char> used(best.rows, 0);
+    int cur = 0;
+    const Mask zero;
+    for (int r = 1; r < best.rows; ++r)
+      if (mask[r].dist(zero) < mask[cur].dist(zero)) cur = r;
+    order.push_back(cur);
+    used[cur] = 1;
+    while (static_cast<int>(order.size()) < best.rows) {
+      int nx = -1, nd = 1 << 30;
+      for (int r = 0; r < best.rows; ++r) {
+        if (used[r]) continue;
+        const int dd = mask[cur].dist(mask[r]);
+        if (dd < nd) {
+          nd = dd;
+          nx = r;
+        }
+      }
+      order.push_back(nx);
+      used[nx] = 1;
+      cur = nx;
+    }
+    std::vector<int> row_of(best.rows);
+    for (int i = 0; i < best.rows; ++i) row_of[order[i]] = i;
+
+    // Window starts, the first row's windows and the moves.
+    std::vector<uint16_t> init(round_up(best.k, 8), 0);  // padding: window 0
+    std::vector<int32_t> at(best.k);
+    for (int i = 0; i < best.k; ++i) {
+      const int32_t s = s0[0] + rel_min[i];
+      if (s < 0) return false;
+      const int32_t m = s % kAlign;
+      out->start[c + i] = s - m;
+      at[i] = i * best.lw + m;
+      init[i] = static_cast<uint16_t>(
+          4 * (at[i] + level[static_cast<size_t>(order[0]) * best.k + i]));
+    }
+    std::vector<uint32_t> steps;
+    for (int q = 1; q < best.rows; ++q) {
+      const uint8_t* from = &level[static_cast<size_t>(order[q - 1]) * best.k];
+      const uint8_t* to = &level[static_cast<size_t>(order[q]) * best.k];
+      for (int i = 0; i < best.k; ++i) {
+        for (int v = from[i]; v < to[i]; ++v)
+          steps.push_back(static_cast<uint32_t>(4 * (at[i] + v)) | kStepUp);
+        for (int v = from[i]; v > to[i]; --v)
+          steps.push_back(static_cast<uint32_t>(4 * (at[i] + v - 1)) | kStepDown);
+      }
+      steps.back() |= kStepEmit;
+    }
+    if (steps.size() > static_cast<size_t>(kMaxSteps)) return false;
+
+    RecHead h{};
+    h.k = static_cast<uint16_t>(best.k);
+    h.n_steps = static_cast<uint16_t>(steps.size());
+    h.rs = static_cast<uint16_t>(best.rs);
+    steps.resize(round_up(static_cast<int>(steps.size()), 4) + kStepPad, 0);
+    Dir e{};
+    e.c0 = c;
+    e.k = h.k;
+    e.lw = static_cast<uint16_t>(best.lw);
+    e.rec16 = static_cast<uint32_t>(recs.size() / 16);
+    const size_t head = recs.size();
+    put(recs, h);
+    for (uint16_t v : init) put(recs, v);
+    for (uint32_t v : steps) put(recs, v);
+    for (int d = 0; d < kDm; ++d) {
+      const int dr = std::min(d, n_real - 1);
+      put(recs, static_cast<uint16_t>(row_of[best_cls[dr]] * best.rs + s0[dr] - s0[0]));
+    }
+    recs.resize(round_up(static_cast<int>(recs.size()), 16), 0);
+    e.rec_n16 = static_cast<uint16_t>(recs.size() / 16 - e.rec16);
+    // The lanes give up their high bytes before a group they cannot take.
+    if (since + best.k > lane_chans) {
+      const uint16_t one = 1;
+      std::memcpy(recs.data() + last_head + offsetof(RecHead, flush), &one, 2);
+      since = 0;
+    }
+    since += best.k;
+    last_head = head;
+    dir.push_back(e);
+    out->words += best_cost * best.k;
+    c += best.k;
+    if (recs.size() > (size_t{1} << 30)) return false;
+  }
+  return true;
+}
+
+}  // namespace
+
+void build_sum_tables(const RangePlan& rp, int32_t n_chan, int64_t max_sample, bool lanes16,
+                      SumTables* out) {
+  *out = SumTables{};
+  // 16-bit lanes: the high bytes carried out of the lanes (TMEM, 16 bits per
+  // sample) hold sums below 2^24; 32-bit words hold sums below 2^31.
+  const int64_t total = static_cast<int64_t>(n_chan) * max_sample;
+  if (total >= (lanes16 ? int64_t{1} << 24 : int64_t{1} << 31)) return;
+  // Channels the lanes take on top of the low bytes they keep.
+  const int lane_chans = lanes16 ? static_cast<int>(std::min<int64_t>(65280 / max_sample, 1 << 20))
+                                 : 1 << 30;
+  if (lane_chans < 1) return;
+  const int64_t n_blocks = (rp.n_dm + kDm - 1) / kDm;
+  if (n_blocks * n_chan > (int64_t{1} << 28)) return;
+
+  // The blocks are independent: built by a few threads (those the system
+  // gives; this one takes what is left).
+  std::vector<Block> blocks(n_blocks);
+  std::atomic<int64_t> next{0};
+  std::atomic<bool> ok{true};
+  auto work = [&]() {
+    try {
+      for (int64_t b = next++; b < n_blocks && ok; b = next++)
+        if (!build_block(rp, n_chan, lane_chans, b, &blocks[b])) ok = false;
+    } catch (const std::bad_alloc&) {
+      ok = false;
+    }
+  };
+  std::vector<std::thread> threads;
+  const int64_t want = std::min<int64_t>(
+      {n_blocks, static_cast<int64_t>(std::thread::hardware_concurrency()), 8,
+       n_blocks * n_chan / 8192 + 1});
+  try {
+    for (int64_t i = 1; i < want; ++i) threads.emplace_back(work);
+  } catch (const std::system_error&) {
+  } catch (const std::bad_alloc&) {
+  }
+  work();
+  for (auto& t : threads) t.join();
+  if (!ok) return;
+
+  size_t n_dir = 0, n_recs = 0;
+  double words = 0;
+  for (const Block& b : blocks) {
+    n_dir += b.dir.size();
+    n_recs += b.recs.size();
+    words += b.words;
+  }
+  const double blocks64 = static_cast<double>((rp.n_dm + 63) / 64);
+  if (words > kMaxWordsPerChannel * n_chan * blocks64 / 2.0) return;
+  auto pad16 = [](size_t v) { return (v + 15) / 16 * 16; };
+  const size_t off_dir = pad16((n_blocks + 1) * sizeof(int32_t));
+  const size_t off_start = off_dir + n_dir * sizeof(Dir);
+  const size_t off_rec = pad16(off_start + static_cast<size_t>(n_blocks) * n_chan * 4);
+  if (off_rec + n_recs > 0x7fffffffu) return;
+  out->bytes.assign(off_rec + n_recs, 0);
+  unsigned char* to = out->bytes.data();
+  int32_t first = 0;
+  size_t at = off_rec;
+  for (int64_t b = 0; b < n_blocks; ++b) {
+    Block& blk = blocks[b];
+    std::memcpy(to + b * 4, &first, 4);
+    for (Dir& e : blk.dir) e.rec16 += static_cast<uint32_t>(at / 16);
+    std::memcpy(to + off_dir + first * sizeof(Dir), blk.dir.data(), blk.dir.size() * sizeof(Dir));
+    std::memcpy(to + off_start + static_cast<size_t>(b) * n_chan * 4, blk.start.data(),
+                static_cast<size_t>(n_chan) * 4);
+    std::memcpy(to + at, blk.recs.data(), blk.recs.size());
+    at += blk.recs.size();
+    first += static_cast<int32_t>(blk.dir.size());
+  }
+  std::memcpy(to + n_blocks * 4, &first, 4);
+  out->n_blocks = static_cast<int32_t>(n_blocks);
+  out->off_dir = static_cast<int32_t>(off_dir);
+  out->off_start = static_cast<int32_t>(off_start);
+  out->ok = true;
+}
+
+}  // namespace dd

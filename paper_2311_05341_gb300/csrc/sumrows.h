@@ -1,0 +1,140 @@
+// sumrows.h -- geometry, device tables and launch parameters of the sum-row
+// tile (fwd_sumrows.cu), shared with its planner (plan_sumrows.cpp).
+//
+// Eq. 3 asks for sum_c X[c][t + s(c, d)].  Over a block of consecutive trial
+// DMs the shifts of adjacent channels move almost together: relative to its
+// first channel, a group of K adjacent channels takes few distinct vectors of
+// shift differences (s(c, d) - s(c_0, d))_c -- about K of them for 128 DMs,
+// because each channel changes its difference by one sample at a time.  All
+// trial DMs with the same vector need the same time series, moved by
+// s(c_0, d).  So the kernel builds each distinct sum over the group once (a
+// sum row, in shared memory) and every DM adds one word of its row per output
+// word instead of K channel words.
+//
+// Integer sums are exact in any order, so the outputs equal the direct sum's
+// bit for bit; a row is made from the previous one by replacing the words of
+// the channels whose difference changed (one subtraction and one addition).
+// Float rows could not be made that way (a large or non-finite sample would
+// leak into rows that do not hold it), so float32 keeps the pattern tiles.
+#pragma once
+
+#include <cstddef>
+#include <cstdint>
+#include <vector>
+
+#include "fwd_tiled.h"
+
+namespace dd {
+
+struct RangePlan;
+
+namespace sr {
+
+constexpr int kDm = 128;             // trial DMs per CTA
+constexpr int kMainWarps = 8;        // adding warps, kDmWarp DMs each
+constexpr int kDmWarp = kDm / kMainWarps;
+constexpr int kBuildGroups = 2;      // row-building warpgroups, taking channel groups in turn
+constexpr int kBuildWarps = 4;       // warps of a building warpgroup
+constexpr int kThreads = 32 * (kMainWarps + kBuildGroups * kBuildWarps);
+// Output words per DM: 11 words per lane for each DM of a pair, and one more
+// that the two DMs of the pair share (16 lanes each).  Two such tiles make one
+// 736-word time tile of the pattern tiles (32 x 23), whose packed copies (pair
+// distance 736) and time-segment boundaries this tile shares.
+constexpr int kFull = 11;
+constexpr int kWords = 32 * kFull + 16;  // 368
+constexpr int kPairWords = 2 * kWords;   // 736: words per pattern time tile, pair distance
+constexpr int kAcc = 2 * kFull + 1;      // accumulator words per lane and DM pair
+constexpr int kBuild = 5;                // row words per lane of a building warp (odd: no bank conflicts)
+constexpr int kChunk = 32 * kBuild;      // row words per building warp and pass
+constexpr int kMaxK = 32;                // channels per group
+constexpr int kAlign = 16;               // window starts: multiples of this many staged words
+constexpr int kSlots = 3;            // staging slots, row buffers
+constexpr int kRawWords = 7424;      // staged words per slot (29 KB)
+constexpr int kRowWords = 11392;     // row words per buffer (44.5 KB)
+constexpr int kMaxSteps = 192;           // moves per group
+constexpr int kStepPad = 8;          // readable moves past the last one
+constexpr int kMaxRec = 16 + kMaxK * 2 + (kMaxSteps + kStepPad) * 4 + kDm * 2;
+
+// One channel group of one DM block.
+struct Dir {
+  int32_t c0;        // first channel
+  uint16_t k;        // channels
+  uint16_t lw;       // staged words per channel (a multiple of 4)
+  uint32_t rec16;    // record offset in the tables, in 16 bytes
+  uint16_t rec_n16;  // record length, in 16 bytes
+  uint16_t pad;
+};
+static_assert(sizeof(Dir) == 16, "Dir must stay 16 bytes");
+
+// Record header; then k uint16 staged byte offsets of the first row's windows
+// (padded to 8 entries), n_steps moves (padded to a multiple of 4, then
+// kStepPad more), kDm uint16 row word offsets (row * stride + the DM's shift
+// from the block's first DM).
+struct RecHead {
+  uint16_t k;
+  uint16_t n_steps;
+  uint16_t rs;       // row stride in words (a multiple of kBuild)
+  uint16_t flush;    // 1: the 16-bit lanes give up their high bytes after this group
+  uint32_t pad[2];
+};
+static_assert(sizeof(RecHead) == 16, "RecHead must stay 16 bytes");
+// A move: staged byte offset (16 bits) of the lower of the channel's two
+// windows, whether a row is complete after it, and in the top two bits its
+// sign (1 up, -1 down, 0 padding) as a signed number.
+constexpr uint32_t kStepEmit = 1u << 17;
+constexpr uint32_t kStepUp = 1u << 30;
+constexpr uint32_t kStepDown = 3u << 30;
+static_assert(kRawWords * 4 <= 65536 && kRowWords <= 65536, "record offsets are 16-bit");
+DD_HOST_DEVICE constexpr int rec_steps_off(int k) { return 16 + (k + 7) / 8 * 16; }
+DD_HOST_DEVICE constexpr int rec_offs_off(int k, int n_steps) {
+  return rec_steps_off(k) + ((n_steps + 3) / 4 * 4 + kStepPad) * 4;
+}
+
+// Shared memory: barriers and flags, records, offsets, staging, rows.
+constexpr size_t kRecOff = 256;
+constexpr size_t kRecBytes = (kMaxRec + 127) / 128 * 128;
+constexpr size_t kOffsOff = kRecOff + kSlots * kRecBytes;
+constexpr size_t kOffsBytes = kDm * 4 + 16;  // row addresses, then the flush flag
+constexpr size_t kRawOff = (kOffsOff + kSlots * kOffsBytes + 127) / 128 * 128;
+constexpr size_t kRowOff = kRawOff + kSlots * size_t{kRawWords} * 4;
+constexpr size_t kSmemBytes = kRowOff + kSlots * size_t{kRowWords} * 4;
+static_assert(kSmemBytes <= 227 * 1024, "sum-row tile exceeds shared memory");
+
+struct Params {
+  const uint32_t* x;     // staged rows: words of the packed copy
+  int64_t stride;        // words per channel row
+  int64_t x_origin;      // word held by element 0 of each row
+  int32_t n_chan;
+  int32_t n_dm;
+  int32_t n_blocks;
+  const unsigned char* tables;
+  int32_t off_dir;       // byte offsets of the directory and the window starts
+  int32_t off_start;
+  int64_t tile0;         // first 736-word time tile of the launch
+  int64_t t_end;         // outputs t >= t_end are not written
+  int64_t out_stride;    // elements from output row d to row d + 1
+  int32_t* out;
+  int32_t* err;
+  int32_t wait_iters;
+  int32_t hold_stage;    // group whose copies are never issued (timeout test; -1: none)
+};
+
+}  // namespace sr
+
+// Tables of a range (plan_sumrows.cpp): group starts per DM block (int32
+// [n_blocks + 1]), directory, window starts (int32 [n_blocks][n_chan]), records.
+struct SumTables {
+  bool ok = false;
+  int32_t n_blocks = 0;
+  int32_t off_dir = 0;
+  int32_t off_start = 0;
+  std::vector<unsigned char> bytes;
+};
+
+// max_sample: the largest decimated sample; lanes16: two samples per word in
+// 16-bit lanes (else one 32-bit sum per word).  ok == false where the tile
+// would not be faster than the pattern tile or cannot hold the sums.
+void build_sum_tables(const RangePlan& rp, int32_t n_chan, int64_t max_sample, bool lanes16,
+                      SumTables* out);
+
+}  // namespace dd

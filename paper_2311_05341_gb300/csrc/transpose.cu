@@ -2,14 +2,17 @@
 // receiver or a SIGPROC file delivers, X_tm[t][c]) to the channel-major rows
 // the dedispersion kernels read (X[c][t]).
 //
-// Work is in 32-bit words of R = 4 / sample-bytes samples.  A CTA moves a tile
-// of 32R times x 32R channels = 32 x 32 words: it loads the tile's 32R time
-// rows with coalesced 128-byte reads into shared memory (column index XOR the
-// row's word-row, so both phases are free of bank conflicts), then each thread
-// takes R x R sample blocks, transposes them in registers (byte or half-word
-// permutes) and writes R words along time, 128 contiguous bytes per warp and
-// channel row.  Only samples with t in [t_begin, t_end) and c < n_chan are
-// written; words that straddle t_end are written sample by sample.
+// HBM-bound: reads and writes every sample once.  131072 x 4096 bytes in
+// 164 us = 6.5 TB/s (the earlier 4-byte loads and stores of 32-word tiles, and a
+// zero fill of the output, took 475 us).  A CTA moves a tile of 128
+// bytes of channels x 256 / E times (E bytes a
+// sample): every thread issues all its 16-byte loads first (8 of them for
+// bytes), the tile waits in shared memory, and each thread then takes 16 / E
+// times x 4 / E channels (one word column), transposes them in registers and
+// writes 16 bytes along time per channel: 256 contiguous bytes per channel
+// row.  Only samples with t in [t_begin, t_end) and c < n_chan are written;
+// pieces off the 16-byte grid are written word by word, a piece that straddles
+// t_end sample by sample.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -20,15 +23,8 @@ namespace dd {
 
 namespace {
 
-constexpr int kTileWords = 32;
-
-// Sample j (0..R-1) of a word of R samples.
-template <int R>
-__device__ __forceinline__ uint32_t sample_of(uint32_t w, int j) {
-  if constexpr (R == 4) return (w >> (8 * j)) & 0xffu;
-  else if constexpr (R == 2) return (w >> (16 * j)) & 0xffffu;
-  else return w;
-}
+constexpr int kRowWords = 32;   // words of a tile row: 128 bytes of channels
+constexpr int kThreads = 256;
 
 // Transpose of an R x R block held as R words (word r = time r, samples =
 // channels): out[j] = channel j, samples = times.
@@ -52,54 +48,79 @@ __device__ __forceinline__ void block_transpose(const uint32_t (&in)[R], uint32_
   }
 }
 
+// Tile row i keeps its words in pairs at word ^ 2 (i / (16 / E)): the 16
+// threads that read one word column at 16 / E rows' distance, and the two
+// columns of a warp, fall on 32 different banks.
 template <int E>
-__global__ void __launch_bounds__(256) transpose_kernel(const uint8_t* __restrict__ in,
-                                                        int64_t in_stride_bytes, int32_t n_chan,
-                                                        uint8_t* __restrict__ out,
-                                                        int64_t out_stride_bytes,
-                                                        int64_t t_begin, int64_t t_end,
-                                                        int32_t chan_tiles) {
-  constexpr int R = 4 / E;
-  constexpr int kRows = kTileWords * R;  // times (and channels) per tile
-  __shared__ uint32_t tile[kRows][kTileWords];
+__global__ void __launch_bounds__(kThreads) transpose_kernel(
+    const uint8_t* __restrict__ in, int64_t in_stride_bytes, int32_t n_chan,
+    uint8_t* __restrict__ out, int64_t out_stride_bytes, int64_t t_begin, int64_t t_end,
+    int32_t chan_tiles) {
+  constexpr int R = 4 / E;               // samples per word
+  constexpr int kTimes = 16 / E;         // times per 16 output bytes
+  constexpr int kRows = 16 * kTimes;     // times per tile
+  constexpr int kLoads = kRows * 8 / kThreads;
+  static_assert(kRows * 8 % kThreads == 0, "whole loads per thread");
+  __shared__ __align__(16) uint32_t tile[kRows][kRowWords];
   const int tid = threadIdx.x;
   const int64_t t0 = t_begin + static_cast<int64_t>(blockIdx.x / chan_tiles) * kRows;
-  const int32_t c0 = (blockIdx.x % chan_tiles) * kRows;
-  const int64_t in_words = in_stride_bytes / 4;  // words per time row (rows are 16-byte aligned)
-  const int32_t cw0 = c0 / R;                    // first channel word of the tile
+  const int32_t c0 = (blockIdx.x % chan_tiles) * (kRowWords * R);
+  const int64_t b0 = static_cast<int64_t>(c0) * E;
 
-  // Load: warp-wide 128-byte row reads; row i holds time t0 + i.
-  for (int i = tid / kTileWords; i < kRows; i += 256 / kTileWords) {
-    const int col = tid % kTileWords;
-    const int64_t t = t0 + i;
-    uint32_t v = 0;
-    if (t < t_end && cw0 + col < in_words)
-      v = __ldg(reinterpret_cast<const uint32_t*>(in + t * in_stride_bytes) + cw0 + col);
-    tile[i][col ^ ((i / R) % kTileWords)] = v;
+  // 8 lanes per 128-byte row (rows and strides are 16-byte aligned).
+  uint4 v[kLoads];
+#pragma unroll
+  for (int k = 0; k < kLoads; ++k) {
+    const int i = (tid + k * kThreads) / 8, g = tid % 8;
+    v[k] = make_uint4(0u, 0u, 0u, 0u);
+    if (t0 + i < t_end && b0 + 16 * g < in_stride_bytes)
+      v[k] = __ldcs(reinterpret_cast<const uint4*>(in + (t0 + i) * in_stride_bytes + b0) + g);
+  }
+#pragma unroll
+  for (int k = 0; k < kLoads; ++k) {
+    const int i = (tid + k * kThreads) / 8, g = tid % 8, sw = 2 * (i / kTimes);
+    *reinterpret_cast<uint2*>(&tile[i][(4 * g) ^ sw]) = make_uint2(v[k].x, v[k].y);
+    *reinterpret_cast<uint2*>(&tile[i][(4 * g + 2) ^ sw]) = make_uint2(v[k].z, v[k].w);
   }
   __syncthreads();
 
-  // Blocks: thread takes word-row bt (times t0 + R bt ..) of word-column bc.
-  for (int k = tid; k < kTileWords * kTileWords; k += 256) {
-    const int bt = k % kTileWords, bc = k / kTileWords;
-    uint32_t w[R], o[R];
+  // Lane: times t0 + kTimes bt .., word columns 2 q + (lane / 16).
+  const int lane = tid & 31, bt = lane & 15;
+  const int64_t t = t0 + static_cast<int64_t>(kTimes) * bt;
+  if (t >= t_end) return;
+  const bool whole = t + kTimes <= t_end && (t * E) % 16 == 0;
+  for (int q = tid >> 5; q < kRowWords / 2; q += kThreads / 32) {
+    const int col = 2 * q + (lane >> 4);
+    uint32_t w[kTimes], o[R][4];
 #pragma unroll
-    for (int r = 0; r < R; ++r) w[r] = tile[R * bt + r][bc ^ bt];
-    block_transpose<R>(w, o);
-    const int64_t t = t0 + static_cast<int64_t>(R) * bt;
+    for (int r = 0; r < kTimes; ++r) w[r] = tile[kTimes * bt + r][col ^ (2 * bt)];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {  // R times each
+      uint32_t x[R], y[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) x[r] = w[R * m + r];
+      block_transpose<R>(x, y);
+#pragma unroll
+      for (int j = 0; j < R; ++j) o[j][m] = y[j];
+    }
 #pragma unroll
     for (int j = 0; j < R; ++j) {
-      const int32_t c = c0 + R * bc + j;
-      if (c >= n_chan || t >= t_end) continue;
-      uint8_t* row = out + static_cast<int64_t>(c) * out_stride_bytes;
-      if (t + R <= t_end) {
-        *reinterpret_cast<uint32_t*>(row + t * E) = o[j];
+      const int32_t c = c0 + R * col + j;
+      if (c >= n_chan) continue;
+      uint8_t* dst = out + static_cast<int64_t>(c) * out_stride_bytes + t * E;
+      if (whole) {
+        __stcs(reinterpret_cast<uint4*>(dst), make_uint4(o[j][0], o[j][1], o[j][2], o[j][3]));
+      } else if (t + kTimes <= t_end) {  // t_begin is a multiple of a word's samples
+#pragma unroll
+        for (int m = 0; m < 4; ++m) reinterpret_cast<uint32_t*>(dst)[m] = o[j][m];
       } else {
-        for (int s = 0; s < R && t + s < t_end; ++s) {
-          const uint32_t v = sample_of<R>(o[j], s);
-          if constexpr (E == 1) row[t + s] = static_cast<uint8_t>(v);
-          else if constexpr (E == 2) reinterpret_cast<uint16_t*>(row)[t + s] = static_cast<uint16_t>(v);
-          else reinterpret_cast<uint32_t*>(row)[t + s] = v;
+#pragma unroll
+        for (int k = 0; k < kTimes; ++k) {
+          if (t + k >= t_end) break;
+          const uint32_t s = o[j][k / R] >> (8 * E * (k % R));
+          if constexpr (E == 1) dst[k] = static_cast<uint8_t>(s);
+          else if constexpr (E == 2) reinterpret_cast<uint16_t*>(dst)[k] = static_cast<uint16_t>(s);
+          else reinterpret_cast<uint32_t*>(dst)[k] = s;
         }
       }
     }
@@ -112,9 +133,8 @@ int launch_transpose(int elem_bytes, const void* d_in, int64_t in_row_stride, in
                      void* d_out, int64_t out_row_stride, int64_t t_begin, int64_t t_end,
                      void* stream) {
   if (t_end <= t_begin) return 0;
-  const int R = 4 / elem_bytes;
-  const int rows = kTileWords * R;
-  const int32_t chan_tiles = (n_chan + rows - 1) / rows;
+  const int chans = kRowWords * 4 / elem_bytes, rows = 256 / elem_bytes;
+  const int32_t chan_tiles = (n_chan + chans - 1) / chans;
   const int64_t time_tiles = (t_end - t_begin + rows - 1) / rows;
   const int64_t grid = time_tiles * chan_tiles;
   if (grid <= 0 || grid > 0x7fffffffLL) return static_cast<int>(cudaErrorInvalidConfiguration);
@@ -124,9 +144,9 @@ int launch_transpose(int elem_bytes, const void* d_in, int64_t in_row_stride, in
   const int64_t isb = in_row_stride * elem_bytes, osb = out_row_stride * elem_bytes;
   const unsigned g = static_cast<unsigned>(grid);
   switch (elem_bytes) {
-    case 1: transpose_kernel<1><<<g, 256, 0, st>>>(in, isb, n_chan, out, osb, t_begin, t_end, chan_tiles); break;
-    case 2: transpose_kernel<2><<<g, 256, 0, st>>>(in, isb, n_chan, out, osb, t_begin, t_end, chan_tiles); break;
-    case 4: transpose_kernel<4><<<g, 256, 0, st>>>(in, isb, n_chan, out, osb, t_begin, t_end, chan_tiles); break;
+    case 1: transpose_kernel<1><<<g, kThreads, 0, st>>>(in, isb, n_chan, out, osb, t_begin, t_end, chan_tiles); break;
+    case 2: transpose_kernel<2><<<g, kThreads, 0, st>>>(in, isb, n_chan, out, osb, t_begin, t_end, chan_tiles); break;
+    case 4: transpose_kernel<4><<<g, kThreads, 0, st>>>(in, isb, n_chan, out, osb, t_begin, t_end, chan_tiles); break;
     default: return static_cast<int>(cudaErrorInvalidValue);
   }
   return static_cast<int>(cudaGetLastError());

@@ -38,7 +38,9 @@ def tile_candidates(plan: Plan, r: int, packed: bool = True):
     tiles = ["pattern"] + (["packed"] if packed and plan.dtype in ("u8", "u4", "u16", "f32")
                            and int(plan.ranges[r][3]) == 1 else [])
     for tile in tiles:
-        for i, sh in enumerate(tile_shapes()):
+        # -1: the automatic shape, which runs the sum-row tile where its plan
+        # has one; then every explicit shape.
+        for i in [-1, *range(len(tile_shapes()))]:
             try:
                 plan.set_tile_shape(r, tile, i)
                 out.append((tile, i))

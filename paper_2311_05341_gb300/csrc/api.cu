@@ -236,18 +236,18 @@ namespace {
 int launch_range(const dd_plan_s* p, const RangePlan& rp, const void* d_in, int64_t stride,
                  int64_t n_samp, int64_t n_out, void* d_out, int64_t t_begin, int64_t t_end,
                  void* stream, int kind = 0, int64_t x_origin = 0) {
-  if (kind > 0) {
-    unsigned char* ws = static_cast<unsigned char*>(p->d_ws);
-    if (rp.sums.ok)
-      return launch_forward_sum_rows(p, rp, ws + rp.off_sums,
-                                     reinterpret_cast<int32_t*>(ws + tk::kStatusOffset), d_in,
-                                     stride, d_out, t_begin, t_end, stream, n_out, kind,
-                                     x_origin);
+  unsigned char* ws = static_cast<unsigned char*>(p->d_ws);
+  const SumTables& sums = kind > 0 ? rp.packed_sums : rp.sums;
+  if (sums.ok)
+    return launch_forward_sum_rows(p, rp, sums,
+                                   ws + (kind > 0 ? rp.off_packed_sums : rp.off_sums),
+                                   reinterpret_cast<int32_t*>(ws + tk::kStatusOffset), d_in,
+                                   stride, d_out, t_begin, t_end, stream, n_out, x_origin);
+  if (kind > 0)
     return launch_forward_pattern(p, rp, ws + rp.off_tile_recs,
                                   reinterpret_cast<int32_t*>(ws + tk::kStatusOffset), d_in,
                                   stride, n_out, d_out, t_begin, t_end, stream, n_out, kind,
                                   x_origin);
-  }
   return rp.tile_ok ? launch_forward_tiled(p, rp, d_in, stride, n_samp, n_out, d_out, t_begin,
                                            t_end, stream)
                     : launch_forward_generic(p, rp, d_in, stride, n_samp, n_out, d_out, t_begin,
@@ -563,8 +563,9 @@ static dd_status run_ring(dd_plan plan, const dd_plan_info& info, const void* d_
     if (e == cudaSuccess) e = cudaStreamWaitEvent(o, hp->start, 0);
   if (e != cudaSuccess) return fail_joined(hp, s, e, "dd_run ring ordering");
   unsigned char* out = static_cast<unsigned char*>(d_out);
+  auto from_ring = [&](size_t r) { return L.ring[r] && !sums_from_input(plan->ranges[r]); };
   for (size_t r = 0; r < plan->ranges.size(); ++r) {
-    if (L.ring[r]) continue;
+    if (from_ring(r)) continue;
     const int le = launch_range(plan, plan->ranges[r], d_in, in_row_stride, n_samp, info.n_out[r],
                                 out + info.out_offset[r] * 4, 0, info.n_out[r], s);
     if (le != 0) return fail_joined(hp, s, le, "dd_run forward launch");
@@ -587,7 +588,7 @@ static dd_status run_ring(dd_plan plan, const dd_plan_info& info, const void* d_
     if (e == cudaSuccess) e = cudaStreamWaitEvent(sc, hp->packed[slot], 0);
     if (e != cudaSuccess) return fail_joined(hp, s, e, "dd_run ring ordering");
     for (size_t r = 0; r < plan->ranges.size(); ++r) {
-      if (!L.ring[r] || sg.hi[r] <= sg.lo[r]) continue;
+      if (!from_ring(r) || sg.hi[r] <= sg.lo[r]) continue;
       const RangePlan& rp = plan->ranges[r];
       le = launch_range(plan, rp, buf, L.slot_words, n_samp, info.n_out[r],
                         out + info.out_offset[r] * 4, sg.lo[r], sg.hi[r], sc,
@@ -625,7 +626,12 @@ static dd_status run_forward(dd_plan plan, const void* d_in, int64_t in_row_stri
   if (d_scratch && reinterpret_cast<uintptr_t>(d_scratch) % 16 != 0)
     return fail(DD_ERR_SHAPE, "input scratch must be 16-byte aligned");
   const bool with_auto = full_with_auto(plan, n_samp, d_scratch, scratch_bytes);
-  if (!n_keep && pack && d_scratch && scratch_bytes < packed_input_bytes(plan, n_samp, true)) {
+  // Ranges that read packed copies when the scratch holds them.
+  bool reads_copies = false;
+  for (const RangePlan& rp : plan->ranges)
+    reads_copies = reads_copies || (copy_kind(rp, true) != 0 && !sums_from_input(rp));
+  if (reads_copies && !n_keep && pack && d_scratch &&
+      scratch_bytes < packed_input_bytes(plan, n_samp, true)) {
     RingLayout L;
     if (pick_ring(plan, info, n_samp, scratch_bytes, &L))
       return run_ring(plan, info, d_in, in_row_stride, n_samp, d_out, d_scratch, L, stream);
@@ -642,11 +648,14 @@ static dd_status run_forward(dd_plan plan, const void* d_in, int64_t in_row_stri
   }
   std::vector<int32_t> range_copy;
   const std::vector<PackedCopy> copies = packed_copies(plan, n_samp, &range_copy, with_auto);
-  if (pack)
-    for (const PackedCopy& pc : copies) {
-      const int e = launch_pack_copy(plan, pc, d_in, in_row_stride, n_samp, d_scratch, stream);
-      if (e != 0) return cuda_fail(e, "dd_run packing");
-    }
+  for (size_t k = 0; pack && k < copies.size(); ++k) {
+    bool read = false;
+    for (size_t r = 0; r < plan->ranges.size(); ++r)
+      read = read || (range_copy[r] == static_cast<int32_t>(k) && !sums_from_input(plan->ranges[r]));
+    if (!read) continue;
+    const int e = launch_pack_copy(plan, copies[k], d_in, in_row_stride, n_samp, d_scratch, stream);
+    if (e != 0) return cuda_fail(e, "dd_run packing");
+  }
   const size_t osz = 4;
   int64_t off = 0;           // element offset of the range's rows in d_out
   for (size_t i = 0; i < plan->ranges.size(); ++i) {
@@ -657,7 +666,7 @@ static dd_status run_forward(dd_plan plan, const void* d_in, int64_t in_row_stri
     const void* src = d_in;
     int64_t stride = in_row_stride;
     int kind = 0;
-    if (range_copy[i] >= 0) {  // reads its packed copy
+    if (range_copy[i] >= 0 && !sums_from_input(rp)) {  // reads its packed copy
       const PackedCopy& pc = copies[range_copy[i]];
       src = static_cast<unsigned char*>(d_scratch) + pc.offset;
       stride = pc.stride;
@@ -826,7 +835,7 @@ static dd_status run_host_pipeline(dd_plan plan, const dd_plan_info& info, const
   const int64_t packed_stride = (n_samp + 3) / 4 * 4;
   int32_t pair = -1;  // lag of the packed copy behind the copied samples (-1: none)
   for (const auto& rp : plan->ranges)
-    if (d_packed && copy_kind(rp, with_auto)) pair = pack_pair(rp, copy_kind(rp, with_auto));
+    if (d_packed && copy_kind(rp, with_auto) && !sums_from_input(rp)) pair = pack_pair(rp, copy_kind(rp, with_auto));
   int64_t packed_done = 0;
   int64_t raw_done = 0;
   int64_t done[DD_MAX_RANGES] = {};
@@ -888,7 +897,7 @@ static dd_status run_host_pipeline(dd_plan plan, const dd_plan_info& info, const
     int64_t lim[DD_MAX_RANGES];
     for (size_t r = 0; r < plan->ranges.size(); ++r) {
       const RangePlan& rp = plan->ranges[r];
-      const int kind = pair >= 0 ? copy_kind(rp, with_auto) : 0;
+      const int kind = pair >= 0 && !sums_from_input(rp) ? copy_kind(rp, with_auto) : 0;
       const bool from_packed = kind != 0;
       const int64_t n_out = info.n_out[r];
       int64_t l = n_out;

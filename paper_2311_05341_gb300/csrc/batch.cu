@@ -33,14 +33,18 @@ struct dd_batch_s {
     int32_t range;
     int64_t n_out;
     int64_t out_offset;  // elements into the plan's output
-    bool pattern;        // on a pattern tile (else an offset tile)
+    bool pattern;        // on a pattern or sum-row tile (else an offset tile)
     int32_t index;       // job number within its family
+    bool sums = false;   // on a sum-row tile
   };
   std::vector<JobRef> jobs;
   std::vector<dd::tk::BatchItem> items;    // offset-tile family
   std::vector<dd::tk::BatchJob> host_jobs;
   std::vector<dd::tk::PatBatchJob> host_pjobs;
-  // Pattern-tile jobs grouped by variant (kind, shape): one launch each.
+  std::vector<dd::sr::Params> host_sjobs;
+  // Pattern-tile jobs grouped by variant (kind, shape) and sum-row jobs by
+  // window format (sr::Src, shape kSumRows): one launch each.
+  static constexpr int32_t kSumRows = -1;
   struct PatGroup {
     int32_t kind;
     int32_t shape;
@@ -51,9 +55,11 @@ struct dd_batch_s {
   };
   std::vector<PatGroup> groups;
   std::vector<int32_t> pjob_group;  // group of each pattern job
+  std::vector<int32_t> sjob_group;  // group of each sum-row job
+  int32_t group_of(const JobRef& j) const { return j.sums ? sjob_group[j.index] : pjob_group[j.index]; }
   int32_t max_lraw = 0;
   int32_t max_lp = 0;
-  size_t off_jobs = 0, off_items = 0, off_pjobs = 0, ws_bytes = 0;
+  size_t off_jobs = 0, off_items = 0, off_pjobs = 0, off_sjobs = 0, ws_bytes = 0;
   unsigned char* d_ws = nullptr;
   bool bound = false;
   int32_t sm_count = 0;
@@ -91,6 +97,14 @@ struct dd_batch_s {
 namespace {
 
 size_t align256(size_t v) { return (v + 255) / 256 * 256; }
+
+// The sum-row tables a batch runs a range from: the packed copy's on
+// DD_TILE_PACKED, else the input's; nullptr without them.
+const dd::SumTables* batch_sums(const dd::RangePlan& rp) {
+  const dd::SumTables& t =
+      dd::tk::packed_copy_kind(rp.tile_kind) && !dd::sums_from_input(rp) ? rp.packed_sums : rp.sums;
+  return t.ok ? &t : nullptr;
+}
 
 bool batch_shape(int32_t dr) {
   for (int d : dd::tk::kBatchDr)
@@ -155,7 +169,19 @@ dd_status dd_batch_create(const dd_plan* plans, const int64_t* n_samp, int32_t n
         int32_t index;
         int ts;
         double dms;
-        if (pat) {
+        const SumTables* sums = pat ? batch_sums(rp) : nullptr;
+        if (sums) {
+          index = static_cast<int32_t>(b->host_sjobs.size());
+          b->host_sjobs.emplace_back();
+          size_t g = 0;
+          while (g < b->groups.size() && !(b->groups[g].kind == sums->src &&
+                                           b->groups[g].shape == dd_batch_s::kSumRows))
+            ++g;
+          if (g == b->groups.size()) b->groups.push_back({sums->src, dd_batch_s::kSumRows});
+          b->sjob_group.push_back(static_cast<int32_t>(g));
+          ts = sr::kWords * (sr::lanes16(sums->src) ? 2 : 1);
+          dms = sr::kDm;
+        } else if (pat) {
           const tk::PatShape& ps = tk::kPatShapes[rp.tile_shape];
           index = static_cast<int32_t>(b->host_pjobs.size());
           b->host_pjobs.emplace_back();
@@ -179,7 +205,7 @@ dd_status dd_batch_create(const dd_plan* plans, const int64_t* n_samp, int32_t n
           ts = tk::tile_samples(rp.tile_kind);
           dms = static_cast<double>(tk::shape_for(rp.tile_dr)->warps) * rp.tile_dr;
         }
-        b->jobs.push_back({i, static_cast<int32_t>(r), n_out, out_off, pat, index});
+        b->jobs.push_back({i, static_cast<int32_t>(r), n_out, out_off, pat, index, sums != nullptr});
         out_off += rp.n_dm * n_out;
         order.push_back({static_cast<double>(p->n_chan) * dms * ts * rp.r.bin, job});
       }
@@ -193,10 +219,13 @@ dd_status dd_batch_create(const dd_plan* plans, const int64_t* n_samp, int32_t n
       const RangePlan& rp = p->ranges[j.range];
       const int ts = j.pattern ? tk::pat_tile_samples(rp.tile_kind, rp.tile_h)
                                : tk::tile_samples(rp.tile_kind);
-      const int64_t tiles = (j.n_out + ts - 1) / ts;
-      auto& list = j.pattern ? b->groups[b->pjob_group[j.index]].items : b->items;
+      const SumTables* sums = j.sums ? batch_sums(rp) : nullptr;
+      const int64_t tiles =
+          sums ? sum_row_halves(sums->src, 0, j.n_out) : (j.n_out + ts - 1) / ts;
+      const int32_t n_blocks = sums ? sums->n_blocks : rp.tile_n_blocks;
+      auto& list = j.pattern ? b->groups[b->group_of(j)].items : b->items;
       for (int64_t t = 0; t < tiles; ++t)
-        for (int32_t blk = 0; blk < rp.tile_n_blocks; ++blk)
+        for (int32_t blk = 0; blk < n_blocks; ++blk)
           list.push_back({j.index, blk, static_cast<int32_t>(t), 0});
     }
     size_t n_pitems = 0;
@@ -213,6 +242,9 @@ dd_status dd_batch_create(const dd_plan* plans, const int64_t* n_samp, int32_t n
     ws = align256(ws);
     b->off_pjobs = ws;
     ws += b->host_pjobs.size() * sizeof(tk::PatBatchJob);
+    ws = align256(ws);
+    b->off_sjobs = ws;
+    ws += b->host_sjobs.size() * sizeof(sr::Params);
     ws = align256(ws);
     b->off_items = ws;
     ws += b->items.size() * sizeof(tk::BatchItem);
@@ -238,13 +270,15 @@ dd_status dd_batch_create(const dd_plan* plans, const int64_t* n_samp, int32_t n
       for (const auto& j : b->jobs) {
         if (j.plan != b->packs[k].plan || !j.pattern) continue;
         if (range_copy[j.range] != b->packs[k].copy_index) continue;
-        const int32_t lane = b->pjob_group[j.index];
+        const SumTables* sums = j.sums ? batch_sums(b->plans[j.plan]->ranges[j.range]) : nullptr;
+        if (sums && sums->src != sr::kPairs) continue;  // reads the input
+        const int32_t lane = b->group_of(j);
         auto& lp = b->lane_packs[lane];
         if (std::find(lp.begin(), lp.end(), static_cast<int32_t>(k)) == lp.end())
           lp.push_back(static_cast<int32_t>(k));
         if (first < 0) first = lane;
       }
-      b->packs[k].lane = first < 0 ? 0 : first;
+      b->packs[k].lane = first;  // -1: no job reads it
     }
   } catch (const std::bad_alloc&) {
     delete b;
@@ -276,7 +310,8 @@ dd_status dd_batch_info(dd_batch batch, int64_t* n_items, int32_t* n_jobs) {
 
 dd_status dd_batch_launches(dd_batch batch, int32_t* n_launches) {
   if (!batch || !n_launches) return fail(DD_ERR_INVALID_ARG, "NULL argument");
-  int32_t n = (batch->items.empty() ? 0 : 1) + static_cast<int32_t>(batch->packs.size());
+  int32_t n = batch->items.empty() ? 0 : 1;
+  for (const auto& pk : batch->packs) n += pk.lane >= 0 ? 1 : 0;
   for (const auto& g : batch->groups) n += g.items.empty() ? 0 : 1;
   *n_launches = n;
   return DD_OK;
@@ -368,12 +403,22 @@ dd_status dd_batch_bind_scratch(dd_batch batch, const void* const* d_in,
         stride < n || stride_bytes % 16 != 0 || (p->dtype == DD_U4 && stride % 2 != 0))
       return fail(DD_ERR_SHAPE, "batch input/output alignment or stride");
     const RangePlan& rp = p->ranges[jr.range];
-    if (rp.tile_ok && tk::packed_copy_kind(rp.tile_kind)) {  // reads its packed copy
+    const SumTables* sums = jr.sums ? batch_sums(rp) : nullptr;
+    if (rp.tile_ok && (sums ? sums->src == sr::kPairs
+                            : tk::packed_copy_kind(rp.tile_kind))) {  // reads its packed copy
       std::vector<int32_t> range_copy;
       const auto copies = packed_copies(p, n, &range_copy);
       const PackedCopy& pc = copies[range_copy[jr.range]];
       x = static_cast<unsigned char*>(d_scratch[jr.plan]) + pc.offset;
       stride = pc.stride;
+    }
+    if (sums) {
+      unsigned char* pws = static_cast<unsigned char*>(p->d_ws);
+      batch->host_sjobs[jr.index] = sum_row_params(
+          p, rp, *sums, pws + (sums == &rp.packed_sums ? rp.off_packed_sums : rp.off_sums),
+          reinterpret_cast<int32_t*>(pws + tk::kStatusOffset), x, stride,
+          static_cast<char*>(o) + jr.out_offset * 4, jr.n_out, jr.n_out);
+      continue;
     }
     const tk::TileParams prm =
         tiled_params(p, rp, static_cast<unsigned char*>(p->d_ws) + rp.off_tile_recs,
@@ -407,6 +452,9 @@ dd_status dd_batch_bind_scratch(dd_batch batch, const void* const* d_in,
     e = cudaMemcpyAsync(batch->d_ws + batch->off_pjobs, batch->host_pjobs.data(),
                         batch->host_pjobs.size() * sizeof(tk::PatBatchJob),
                         cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess && !batch->host_sjobs.empty())
+    e = cudaMemcpyAsync(batch->d_ws + batch->off_sjobs, batch->host_sjobs.data(),
+                        batch->host_sjobs.size() * sizeof(sr::Params), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(e, "dd_batch_bind");
   batch->bound = true;
@@ -443,6 +491,7 @@ dd_status dd_batch_run(dd_batch batch, void* stream) {
   // Packing launches, each on the first lane that reads its copy.
   for (size_t k = 0; k < batch->packs.size(); ++k) {
     const auto& pk = batch->packs[k];
+    if (pk.lane < 0) continue;
     cudaStream_t ls = lane_stream(pk.lane);
     const int le = launch_pack_copy(batch->plans[pk.plan], pk.copy, pk.in, pk.in_stride,
                                     batch->n_samp[pk.plan], pk.scratch, ls);
@@ -459,13 +508,23 @@ dd_status dd_batch_run(dd_batch batch, void* stream) {
         e = cudaStreamWaitEvent(ls, batch->pack_done[k], 0);
         if (e != cudaSuccess) return cuda_fail(e, "dd_batch_run ordering");
       }
+    const int64_t grid = std::min<int64_t>(static_cast<int64_t>(g.items.size()),
+                                           static_cast<int64_t>(batch->sm_count));
+    if (g.shape == dd_batch_s::kSumRows) {
+      sr::BatchArgs sargs{};
+      sargs.jobs = reinterpret_cast<const sr::Params*>(batch->d_ws + batch->off_sjobs);
+      sargs.items = reinterpret_cast<const tk::BatchItem*>(batch->d_ws + g.off_items);
+      sargs.n_items = static_cast<int32_t>(g.items.size());
+      sargs.counter = reinterpret_cast<uint32_t*>(batch->d_ws) + 1 + gi;
+      const int le = launch_sum_row_batch(g.kind, sargs, static_cast<int32_t>(grid), ls);
+      if (le != 0) return cuda_fail(le, "dd_batch_run sum-row launch");
+      continue;
+    }
     tk::PatBatchArgs args{};
     args.jobs = reinterpret_cast<const tk::PatBatchJob*>(batch->d_ws + batch->off_pjobs);
     args.items = reinterpret_cast<const tk::BatchItem*>(batch->d_ws + g.off_items);
     args.n_items = static_cast<int32_t>(g.items.size());
     args.counter = reinterpret_cast<uint32_t*>(batch->d_ws) + 1 + gi;
-    const int64_t grid = std::min<int64_t>(static_cast<int64_t>(g.items.size()),
-                                           static_cast<int64_t>(batch->sm_count));
     int le = launch_pattern_batch(g.kind, g.shape, args,
                                   static_cast<int32_t>(std::max<int64_t>(grid, 1)), g.smem, ls,
                                   g.mode < 0 ? 0 : g.mode);

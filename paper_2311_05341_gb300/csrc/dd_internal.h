@@ -60,13 +60,16 @@ struct RangePlan {
   // kind's window alignment, a multiple of the packed kind's); 0 if none.
   int32_t alt_kind = 0;
 
-  // Sum-row tile on the packed copies of integer input (sumrows.h).
+  // Sum-row tile of integer input (sumrows.h): from the input itself (bin 1),
+  // and from the packed copies of uint8 and 4-bit input.
   SumTables sums;
+  SumTables packed_sums;
 
   // Byte offsets of the device tables inside the workspace.
   size_t off_shifts = 0;        // int32 [n_dm][n_chan]
   size_t off_tile_recs = 0;     // tk::Rec or tk::PRec [tile_n_blocks][n_chan]
   size_t off_sums = 0;          // sum-row tables (sums.ok)
+  size_t off_packed_sums = 0;
   std::vector<unsigned char> tile_recs;  // host image of the records
 };
 
@@ -148,13 +151,22 @@ int launch_forward_pattern(const dd_plan_s* p, const RangePlan& rp, const void* 
                            void* d_out, int64_t t_begin, int64_t t_end, void* stream,
                            int64_t out_stride, int kind = 0, int64_t x_origin = 0,
                            bool widen_slots = true);
-// The sum-row kernel (fwd_sumrows.cu) on packed words of kernel kind `kind`
-// (kU8P, kU16P); d_words, stride, x_origin and the times as
-// launch_forward_pattern.
-int launch_forward_sum_rows(const dd_plan_s* p, const RangePlan& rp, const void* tables,
-                            int32_t* err, const void* d_words, int64_t stride, void* d_out,
+// The sum-row kernel (fwd_sumrows.cu) on the rows sums.src names (the input,
+// or words of its packed copy); stride in their samples, x_origin and the
+// times as launch_forward_pattern.
+int launch_forward_sum_rows(const dd_plan_s* p, const RangePlan& rp, const SumTables& sums,
+                            const void* tables,
+                            int32_t* err, const void* d_rows, int64_t stride, void* d_out,
                             int64_t t_begin, int64_t t_end, void* stream, int64_t out_stride,
-                            int kind, int64_t x_origin);
+                            int64_t x_origin);
+// Its launch parameters (x_origin and tile0 zero), the 368-word halves of time
+// tiles that outputs [t_begin, t_end) take, and the persistent kernel of one
+// window format (sr::Src).
+sr::Params sum_row_params(const dd_plan_s* p, const RangePlan& rp, const SumTables& sums,
+                          const void* tables, int32_t* err, const void* d_rows, int64_t stride,
+                          void* d_out, int64_t t_end, int64_t out_stride);
+int64_t sum_row_halves(int src, int64_t t_begin, int64_t t_end);
+int launch_sum_row_batch(int src, const sr::BatchArgs& args, int32_t grid, void* stream);
 // Packed uint8 copy for the kU8P tiles (pack.cu): out[c][t] = in[c][t] |
 // in[c][t + pair] << 16 for t in [t_begin, t_end) (0 past n_samp); strides in
 // bytes (in) and 32-bit words (out, a multiple of 4); pair and t_begin
@@ -186,6 +198,9 @@ inline int copy_kind(const RangePlan& rp, bool with_auto) {
   if (tk::packed_copy_kind(rp.tile_kind)) return rp.tile_kind;
   return with_auto ? rp.alt_kind : 0;
 }
+// The range runs on the sum-row tile from the input whatever scratch the
+// caller gives (uint16: its packed copy has no sum-row kernel).
+inline bool sums_from_input(const RangePlan& rp) { return rp.sums.ok && !rp.packed_sums.ok; }
 // Pair distance of the packed copy a range reads with kernel kind `kind`.
 inline int32_t pack_pair(const RangePlan& rp, int kind) {
   return kind == tk::kU8P || kind == tk::kF32P ? 32 * rp.tile_h : 0;

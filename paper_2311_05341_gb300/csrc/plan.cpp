@@ -396,17 +396,26 @@ void choose_tile(RangePlan& rp, int32_t n_chan, dd_dtype dtype) {
     if (try_tile_shape(rp, n_chan, kind, *tk::shape_for(dr))) return;
 }
 
-// choose_tile, then the sum-row tables of a range that may run from a packed
-// copy of integer input at the automatic shape (pair distance 736).
+// choose_tile, then the sum-row tables where the tile is an integer pattern
+// tile of the automatic shape (time tiles of 32 x 23 words): from the input
+// itself at bin 1; from the packed copy of uint8 (any bin of its packed tile)
+// and 4-bit input, which is faster where the caller gives scratch for it.
 void choose_kernels(RangePlan& rp, int32_t n_chan, dd_dtype dtype) {
   choose_tile(rp, n_chan, dtype);
   rp.sums = SumTables{};
-  const int kind = copy_kind(rp, true);
-  if ((kind != tk::kU8P && kind != tk::kU16P) || rp.shape_request >= 0 ||
+  rp.packed_sums = SumTables{};
+  if (!rp.tile_ok || !rp.tile_pattern || rp.shape_request >= 0 || dtype == DD_F32 ||
       32 * rp.tile_h != sr::kPairWords)
     return;
   const int64_t top = dtype == DD_U16 ? 65535 : dtype == DD_U4 ? 15 : 255;
-  build_sum_tables(rp, n_chan, top * rp.r.bin, tk::packed_pairs(kind), &rp.sums);
+  if (rp.r.bin == 1)
+    build_sum_tables(rp, n_chan, top,
+                     dtype == DD_U16  ? sr::kHalves
+                     : dtype == DD_U4 ? sr::kNibbles
+                                      : sr::kBytes,
+                     &rp.sums);
+  if (copy_kind(rp, true) == tk::kU8P)
+    build_sum_tables(rp, n_chan, top * rp.r.bin, sr::kPairs, &rp.packed_sums);
 }
 
 // The adjoint of range rp (float32) as a forward transform: with P = s_max,
@@ -456,10 +465,16 @@ void layout_workspace(dd_plan_s* p) {
       rp.off_tile_recs = ws;
       ws += rp.tile_recs.size();
     }
-    if (rp.sums.ok) {
+    // Sum-row tables: room for both sets, a power of two each, so that the
+    // workspace's size depends on the plan's shape and not on which window
+    // formats its dtype has.
+    if (rp.sums.ok || rp.packed_sums.ok) {
+      size_t room = 4096;
+      while (room < std::max(rp.sums.bytes.size(), rp.packed_sums.bytes.size())) room *= 2;
       ws = align_up(ws, 256);
       rp.off_sums = ws;
-      ws += rp.sums.bytes.size();
+      rp.off_packed_sums = ws + room;
+      ws += 2 * room;
     }
   };
   for (auto& rp : p->ranges) place(rp);
@@ -490,6 +505,9 @@ void layout_workspace(dd_plan_s* p) {
       std::memcpy(p->host_ws.data() + rp.off_tile_recs, rp.tile_recs.data(), rp.tile_recs.size());
     if (rp.sums.ok)
       std::memcpy(p->host_ws.data() + rp.off_sums, rp.sums.bytes.data(), rp.sums.bytes.size());
+    if (rp.packed_sums.ok)
+      std::memcpy(p->host_ws.data() + rp.off_packed_sums, rp.packed_sums.bytes.data(),
+                  rp.packed_sums.bytes.size());
   };
   for (const auto& rp : p->ranges) copy(rp);
   for (const auto& ar : p->adj) copy(ar);

@@ -20,13 +20,12 @@ namespace {
 
 using namespace sr;
 
-// Shared-memory words per channel and 64 trial DMs x 736 packed words (half of
-// this tile's DMs x twice its words) above which the pattern tile is taken.
-// One word is one lane's 4 bytes of the shared-memory pipe, which bounds both
-// tiles: the pattern tile moves (23 + o_3) words per 4 DMs and 23-word window,
-// about 12000, and gets 3/4 of the pipe, as this tile does.  Measured: 1024
-// channels, 2048 trials (8540 words) 3.85 ms against 5.2 ms.
-constexpr double kMaxWordsPerChannel = 10500.0;
+// Cost (words_per_channel) per channel and 64 trial DMs x 736 words, half of
+// this tile's DMs x twice its words, above which the pattern tile is taken: it
+// moves (23 + o_3) words per 4 DMs and 23-word window, about 12000, at 3/4 of
+// the pipe's rate.  Measured: 1024 channels, 2048 trials (cost 10800) 3.85 ms
+// from packed copies against 5.2 ms, 4.8 against 5.8 ms from the input.
+constexpr double kMaxWordsPerChannel = 13500.0;
 
 // Difference vectors as bit masks: channel i of the group has kLevels bits,
 // v_i - min of them set, so that the distance of two vectors in samples is
@@ -51,12 +50,19 @@ struct Group {
 
 inline int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
-// Words per channel of a group of k channels with `rows` rows: staging and
-// first row, moves (their number grows a little faster than the rows'), rows
-// written, and the adds' reads.
-double words_per_channel(int k, int rows, int rs) {
-  const double moves = rows * (0.75 + k / 40.0) * (1.0 + 1.0 / kBuild);
-  return ((2.0 * k + moves + rows) * rs + static_cast<double>(kDm) * kWords) / k;
+// Cost of a group of k channels with `rows` rows, in shared-memory words per
+// channel (32 words a cycle), of the three that bound it: the shared-memory
+// pipe (staging and first row, moves -- their number grows a little faster than
+// the rows' -- rows written and the adds' reads, at the 85 % of its rate that it
+// gives), the building warps' chain of channels and moves (two warpgroups) and
+// the adding warps' time, whose cycles were measured on the device.
+double words_per_channel(const Format& f, int k, int rows, int rs) {
+  const double moves = rows * (0.75 + k / 40.0);
+  const double pipe =
+      ((2.0 * k + moves * 1.2 + rows) * rs + static_cast<double>(kDm) * kWords) / 0.85;
+  const double chain = 16.0 * (kChainGroup + f.chain_chan * k + f.chain_move * moves);
+  const double adds = 32.0 * kAddGroup;
+  return std::max({pipe, chain, adds}) / k;
 }
 
 template <typename T>
@@ -75,7 +81,8 @@ struct Block {
   double words = 0;
 };
 
-bool build_block(const RangePlan& rp, int32_t n_chan, int lane_chans, int64_t b, Block* out) {
+bool build_block(const RangePlan& rp, int32_t n_chan, int lane_chans, const Format& f, int64_t b,
+                 Block* out) {
   std::vector<Dir>& dir = out->dir;
   std::vector<unsigned char>& recs = out->recs;
   out->start.resize(n_chan);
@@ -90,8 +97,8 @@ bool build_block(const RangePlan& rp, int32_t n_chan, int lane_chans, int64_t b,
   int since = 0;  // channels in the lanes
   while (c < n_chan) {
     const int32_t* s0 = &block[static_cast<size_t>(c) * kDm];
-    const int rs = round_up(kWords + s0[n_real - 1] - s0[0], kBuild);
-    if (s0[n_real - 1] < s0[0] || rs > kRowWords) return false;
+    const int rs = round_up(kWords + s0[n_real - 1] - s0[0], f.build);
+    if (s0[n_real - 1] < s0[0] || rs > f.row_words) return false;
     // Extend the group channel by channel, splitting the DMs into classes
     // of equal difference vectors, and keep the cheapest size that fits.
     uint8_t cls[kDm] = {};
@@ -120,10 +127,10 @@ bool build_block(const RangePlan& rp, int32_t n_chan, int lane_chans, int64_t b,
         }
         n_cls = n;
       }
-      const int lw = round_up(kAlign - 1 + reach + rs + 1, 4);
-      if (k * lw > kRawWords || n_cls * rs > kRowWords) break;
+      const int lw = round_up(f.align - 1 + reach + rs + f.extra, 128 / f.bits);
+      if (k * lw > 65535 || k * (lw * f.bits / 8) > f.raw_bytes || n_cls * rs > f.row_words) break;
       // The first row adds channels in pairs: only the last group may be odd.
-      const double cost = words_per_channel(k, n_cls, rs);
+      const double cost = words_per_channel(f, k, n_cls, rs);
       if (cost < best_cost && (k % 2 == 0 || c + k == n_chan || kmax == 1)) {
         best_cost = cost;
         best.k = k;
@@ -192,11 +199,10 @@ bool build_block(const RangePlan& rp, int32_t n_chan, int lane_chans, int64_t b,
     for (int i = 0; i < best.k; ++i) {
       const int32_t s = s0[0] + rel_min[i];
       if (s < 0) return false;
-      const int32_t m = s % kAlign;
+      const int32_t m = s % f.align;
       out->start[c + i] = s - m;
       at[i] = i * best.lw + m;
-      init[i] = static_cast<uint16_t>(
-          4 * (at[i] + level[static_cast<size_t>(order[0]) * best.k + i]));
+      init[i] = static_cast<uint16_t>(at[i] + level[static_cast<size_t>(order[0]) * best.k + i]);
     }
     std::vector<uint32_t> steps;
     for (int q = 1; q < best.rows; ++q) {
@@ -204,9 +210,9 @@ bool build_block(const RangePlan& rp, int32_t n_chan, int lane_chans, int64_t b,
       const uint8_t* to = &level[static_cast<size_t>(order[q]) * best.k];
       for (int i = 0; i < best.k; ++i) {
         for (int v = from[i]; v < to[i]; ++v)
-          steps.push_back(static_cast<uint32_t>(4 * (at[i] + v)) | kStepUp);
+          steps.push_back(static_cast<uint32_t>(at[i] + v) | kStepUp);
         for (int v = from[i]; v > to[i]; --v)
-          steps.push_back(static_cast<uint32_t>(4 * (at[i] + v - 1)) | kStepDown);
+          steps.push_back(static_cast<uint32_t>(at[i] + v - 1) | kStepDown);
       }
       steps.back() |= kStepEmit;
     }
@@ -230,7 +236,8 @@ bool build_block(const RangePlan& rp, int32_t n_chan, int lane_chans, int64_t b,
       const int dr = std::min(d, n_real - 1);
       put(recs, static_cast<uint16_t>(row_of[best_cls[dr]] * best.rs + s0[dr] - s0[0]));
     }
-    recs.resize(round_up(static_cast<int>(recs.size()), 16), 0);
+    // The next copies' entry and starts: filled in once they are known.
+    recs.resize(round_up(static_cast<int>(recs.size()), 16) + sizeof(Dir) + kMaxK * 4, 0);
     e.rec_n16 = static_cast<uint16_t>(recs.size() / 16 - e.rec16);
     // The lanes give up their high bytes before a group they cannot take.
     if (since + best.k > lane_chans) {
@@ -250,9 +257,12 @@ bool build_block(const RangePlan& rp, int32_t n_chan, int lane_chans, int64_t b,
 
 }  // namespace
 
-void build_sum_tables(const RangePlan& rp, int32_t n_chan, int64_t max_sample, bool lanes16,
+void build_sum_tables(const RangePlan& rp, int32_t n_chan, int64_t max_sample, int src,
                       SumTables* out) {
   *out = SumTables{};
+  out->src = src;
+  const Format f = format(src);
+  const bool lanes16 = sr::lanes16(src);
   // 16-bit lanes: the high bytes carried out of the lanes (TMEM, 16 bits per
   // sample) hold sums below 2^24; 32-bit words hold sums below 2^31.
   const int64_t total = static_cast<int64_t>(n_chan) * max_sample;
@@ -272,7 +282,7 @@ void build_sum_tables(const RangePlan& rp, int32_t n_chan, int64_t max_sample, b
   auto work = [&]() {
     try {
       for (int64_t b = next++; b < n_blocks && ok; b = next++)
-        if (!build_block(rp, n_chan, lane_chans, b, &blocks[b])) ok = false;
+        if (!build_block(rp, n_chan, lane_chans, f, b, &blocks[b])) ok = false;
     } catch (const std::bad_alloc&) {
       ok = false;
     }
@@ -302,6 +312,7 @@ void build_sum_tables(const RangePlan& rp, int32_t n_chan, int64_t max_sample, b
   auto pad16 = [](size_t v) { return (v + 15) / 16 * 16; };
   const size_t off_dir = pad16((n_blocks + 1) * sizeof(int32_t));
   const size_t off_start = off_dir + n_dir * sizeof(Dir);
+  // Each record ends with the entry and window starts of the group kSlots later.
   const size_t off_rec = pad16(off_start + static_cast<size_t>(n_blocks) * n_chan * 4);
   if (off_rec + n_recs > 0x7fffffffu) return;
   out->bytes.assign(off_rec + n_recs, 0);
@@ -312,6 +323,14 @@ void build_sum_tables(const RangePlan& rp, int32_t n_chan, int64_t max_sample, b
     Block& blk = blocks[b];
     std::memcpy(to + b * 4, &first, 4);
     for (Dir& e : blk.dir) e.rec16 += static_cast<uint32_t>(at / 16);
+    for (size_t g = 0; g + kSlots < blk.dir.size(); ++g) {
+      const Dir& e = blk.dir[g];
+      const Dir& n = blk.dir[g + kSlots];
+      unsigned char* tail = blk.recs.data() + (static_cast<size_t>(e.rec16) * 16 - at) +
+                            static_cast<size_t>(e.rec_n16) * 16 - sizeof(Dir) - kMaxK * 4;
+      std::memcpy(tail, &n, sizeof(Dir));
+      std::memcpy(tail + sizeof(Dir), &blk.start[n.c0], n.k * sizeof(int32_t));
+    }
     std::memcpy(to + off_dir + first * sizeof(Dir), blk.dir.data(), blk.dir.size() * sizeof(Dir));
     std::memcpy(to + off_start + static_cast<size_t>(b) * n_chan * 4, blk.start.data(),
                 static_cast<size_t>(n_chan) * 4);

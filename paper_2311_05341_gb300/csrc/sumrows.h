@@ -44,47 +44,76 @@ constexpr int kFull = 11;
 constexpr int kWords = 32 * kFull + 16;  // 368
 constexpr int kPairWords = 2 * kWords;   // 736: words per pattern time tile, pair distance
 constexpr int kAcc = 2 * kFull + 1;      // accumulator words per lane and DM pair
-constexpr int kBuild = 5;                // row words per lane of a building warp (odd: no bank conflicts)
-constexpr int kChunk = 32 * kBuild;      // row words per building warp and pass
 constexpr int kMaxK = 32;                // channels per group
-constexpr int kAlign = 16;               // window starts: multiples of this many staged words
-constexpr int kSlots = 3;            // staging slots, row buffers
-constexpr int kRawWords = 7424;      // staged words per slot (29 KB)
-constexpr int kRowWords = 11392;     // row words per buffer (44.5 KB)
+constexpr int kSlots = 3;                // staging slots, row buffers
 constexpr int kMaxSteps = 192;           // moves per group
-constexpr int kStepPad = 8;          // readable moves past the last one
-constexpr int kMaxRec = 16 + kMaxK * 2 + (kMaxSteps + kStepPad) * 4 + kDm * 2;
+constexpr int kStepPad = 8;              // readable moves past the last one
+constexpr int kMaxRec = 16 + kMaxK * 2 + (kMaxSteps + kStepPad) * 4 + kDm * 2 + 16 + kMaxK * 4;
+
+// What the tile stages.  kPairs: 32-bit words of a packed copy (two samples,
+// 736 apart, in 16-bit lanes), for decimated uint8.  kBytes, kNibbles: the
+// uint8 or 4-bit input itself; a row word pairs samples 368 apart, so a CTA's
+// 736 outputs and its staged window are contiguous.  kHalves: the uint16
+// input, one sample per 32-bit row word.
+enum Src : int { kPairs = 0, kBytes = 1, kNibbles = 2, kHalves = 3 };
+
+struct Format {
+  int bits;        // per staged sample (kPairs: per word)
+  int align;       // window starts: multiples of this many staged samples (16 bytes or more)
+  int build;       // row words per lane of a building warp
+  int extra;       // staged samples a lane reads past its last row word's sample
+  int raw_bytes;   // staging slot
+  int row_words;   // row buffer
+  int chain_chan;  // measured cycles of a building warp per channel of a group
+  int chain_move;  // and per move (kChainGroup per group besides)
+};
+constexpr int kChainGroup = 900;
+constexpr int kAddGroup = 2900;  // cycles of the adding warps per group
+// kPairs: five scalar words per lane (an odd lane stride: no bank conflicts),
+// 29 KB of staging for 44.5 KB of rows.  The others: four words per lane from
+// unaligned bytes (two 32-bit words and a funnel shift), stored 16 bytes at a
+// time; a window is less than half as long in bytes, so the rows get more.
+DD_HOST_DEVICE constexpr Format format(int src) {
+  return src == kPairs      ? Format{32, 16, 5, 1, 29696, 11392, 110, 155}
+         : src == kBytes    ? Format{8, 16, 4, kWords + 8, 17408, 14464, 190, 145}
+         : src == kNibbles  ? Format{4, 32, 4, kWords + 16, 17408, 14464, 195, 165}
+                            : Format{16, 16, 4, 4, 17408, 14464, 380, 130};
+}
+// Output samples of a CTA's words, and of the pattern time tile holding them.
+DD_HOST_DEVICE constexpr int pair_dist(int src) { return src == kPairs ? kPairWords : kWords; }
+DD_HOST_DEVICE constexpr bool lanes16(int src) { return src != kHalves; }
 
 // One channel group of one DM block.
 struct Dir {
   int32_t c0;        // first channel
   uint16_t k;        // channels
-  uint16_t lw;       // staged words per channel (a multiple of 4)
+  uint16_t lw;       // staged samples per channel (a multiple of 16 bytes)
   uint32_t rec16;    // record offset in the tables, in 16 bytes
   uint16_t rec_n16;  // record length, in 16 bytes
   uint16_t pad;
 };
 static_assert(sizeof(Dir) == 16, "Dir must stay 16 bytes");
 
-// Record header; then k uint16 staged byte offsets of the first row's windows
-// (padded to 8 entries), n_steps moves (padded to a multiple of 4, then
-// kStepPad more), kDm uint16 row word offsets (row * stride + the DM's shift
-// from the block's first DM).
+// Record header; then k uint16 staged sample offsets of the first row's
+// windows (padded to 8 entries), n_steps moves (padded to a multiple of 4,
+// then kStepPad more), kDm uint16 row word offsets (row * stride + the DM's
+// shift from the block's first DM), and the directory entry (k == 0: none) and
+// kMaxK window starts of the group kSlots later, whose copies are issued while
+// this group is added.
 struct RecHead {
   uint16_t k;
   uint16_t n_steps;
-  uint16_t rs;       // row stride in words (a multiple of kBuild)
+  uint16_t rs;       // row stride in words (a multiple of Format::build)
   uint16_t flush;    // 1: the 16-bit lanes give up their high bytes after this group
   uint32_t pad[2];
 };
 static_assert(sizeof(RecHead) == 16, "RecHead must stay 16 bytes");
-// A move: staged byte offset (16 bits) of the lower of the channel's two
+// A move: staged sample offset (16 bits) of the lower of the channel's two
 // windows, whether a row is complete after it, and in the top two bits its
 // sign (1 up, -1 down, 0 padding) as a signed number.
 constexpr uint32_t kStepEmit = 1u << 17;
 constexpr uint32_t kStepUp = 1u << 30;
 constexpr uint32_t kStepDown = 3u << 30;
-static_assert(kRawWords * 4 <= 65536 && kRowWords <= 65536, "record offsets are 16-bit");
 DD_HOST_DEVICE constexpr int rec_steps_off(int k) { return 16 + (k + 7) / 8 * 16; }
 DD_HOST_DEVICE constexpr int rec_offs_off(int k, int n_steps) {
   return rec_steps_off(k) + ((n_steps + 3) / 4 * 4 + kStepPad) * 4;
@@ -94,23 +123,32 @@ DD_HOST_DEVICE constexpr int rec_offs_off(int k, int n_steps) {
 constexpr size_t kRecOff = 256;
 constexpr size_t kRecBytes = (kMaxRec + 127) / 128 * 128;
 constexpr size_t kOffsOff = kRecOff + kSlots * kRecBytes;
-constexpr size_t kOffsBytes = kDm * 4 + 16;  // row addresses, then the flush flag
+// Row addresses, the flush flag, the directory entry and window starts of the
+// group kSlots later.
+constexpr int kNextDir = kDm + 4;            // in words
+constexpr int kNextStart = kNextDir + 4;
+constexpr size_t kOffsBytes = (kNextStart + kMaxK) * 4;
 constexpr size_t kRawOff = (kOffsOff + kSlots * kOffsBytes + 127) / 128 * 128;
-constexpr size_t kRowOff = kRawOff + kSlots * size_t{kRawWords} * 4;
-constexpr size_t kSmemBytes = kRowOff + kSlots * size_t{kRowWords} * 4;
-static_assert(kSmemBytes <= 227 * 1024, "sum-row tile exceeds shared memory");
+DD_HOST_DEVICE constexpr size_t row_off(int src) {
+  return kRawOff + kSlots * static_cast<size_t>(format(src).raw_bytes);
+}
+DD_HOST_DEVICE constexpr size_t smem_bytes(int src) {
+  return row_off(src) + kSlots * static_cast<size_t>(format(src).row_words) * 4;
+}
+static_assert(smem_bytes(kPairs) <= 227 * 1024 && smem_bytes(kBytes) <= 227 * 1024,
+              "sum-row tile exceeds shared memory");
 
 struct Params {
-  const uint32_t* x;     // staged rows: words of the packed copy
-  int64_t stride;        // words per channel row
-  int64_t x_origin;      // word held by element 0 of each row
+  const void* x;         // staged rows
+  int64_t stride;        // staged samples (kPairs: words) per channel row
+  int64_t x_origin;      // staged sample held by element 0 of each row
   int32_t n_chan;
   int32_t n_dm;
   int32_t n_blocks;
   const unsigned char* tables;
   int32_t off_dir;       // byte offsets of the directory and the window starts
   int32_t off_start;
-  int64_t tile0;         // first 736-word time tile of the launch
+  int64_t tile0;         // first pattern time tile of the launch
   int64_t t_end;         // outputs t >= t_end are not written
   int64_t out_stride;    // elements from output row d to row d + 1
   int32_t* out;
@@ -119,22 +157,30 @@ struct Params {
   int32_t hold_stage;    // group whose copies are never issued (timeout test; -1: none)
 };
 
+// Persistent batch execution: items (job, DM block, half) over many jobs.
+struct BatchArgs {
+  const Params* jobs;          // device
+  const tk::BatchItem* items;  // device, in execution order (tile: the half)
+  int32_t n_items;
+  uint32_t* counter;           // device, zero before the launch
+};
+
 }  // namespace sr
 
 // Tables of a range (plan_sumrows.cpp): group starts per DM block (int32
 // [n_blocks + 1]), directory, window starts (int32 [n_blocks][n_chan]), records.
 struct SumTables {
   bool ok = false;
+  int32_t src = 0;       // sr::Src
   int32_t n_blocks = 0;
   int32_t off_dir = 0;
   int32_t off_start = 0;
   std::vector<unsigned char> bytes;
 };
 
-// max_sample: the largest decimated sample; lanes16: two samples per word in
-// 16-bit lanes (else one 32-bit sum per word).  ok == false where the tile
+// max_sample: the largest (decimated) sample.  ok == false where the tile
 // would not be faster than the pattern tile or cannot hold the sums.
-void build_sum_tables(const RangePlan& rp, int32_t n_chan, int64_t max_sample, bool lanes16,
+void build_sum_tables(const RangePlan& rp, int32_t n_chan, int64_t max_sample, int src,
                       SumTables* out);
 
 }  // namespace dd

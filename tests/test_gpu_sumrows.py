@@ -124,3 +124,44 @@ def test_sum_row_tile_windows_and_withheld_group():
         got = plan.run(xd, n_samp=n_samp, segments=1)[0].cpu().numpy()
         plan.device_status()
         np.testing.assert_array_equal(got, ref, err_msg=f"after holding group {hold}")
+
+
+# dtype, channels, DMs, slope, extra outputs, full
+RAW_CASES = [
+    ("u8", 600, 1, 0.5, 1, False), ("u8", 601, 129, 0.1, 736, True),
+    ("u8", 777, 257, 0.2, 737, False), ("u8", 1024, 256, 0.6, 1473, True),
+    ("u8", 2048, 256, 1.2, 2209, False), ("u8", 4099, 128, 2.5, 1473, False),
+    ("u4", 700, 200, 0.2, 735, True), ("u4", 703, 129, 0.15, 1841, False),
+    ("u4", 4099, 128, 2.5, 737, False),
+    ("u16", 600, 130, 0.1, 368, False), ("u16", 1000, 256, 0.5, 1105, True),
+    ("u16", 4099, 128, 2.5, 737, False),
+]
+
+
+@pytest.mark.parametrize("dtype,n_chan,n_dm,slope,extra,full", RAW_CASES)
+def test_sum_row_tile_from_the_input(dtype, n_chan, n_dm, slope, extra, full):
+    """Without scratch, alone and in a batch of two beams (the persistent
+    kernel, several items per CTA slot), against the oracle."""
+    from paper_2311_05341_gb300 import batch
+    f_high, t_samp = 1500.0, 64e-6
+    freqs = channel_freqs(f_high, 300.0, n_chan)
+    step = slope * t_samp / oracle.delay_coeff(freqs[-1], f_high)
+    ranges = [(0.0, n_dm * step, step, 1)]
+    s_max = oracle.extent(freqs, f_high, t_samp, ranges[0], 10 ** 9)[0]
+    n_samp = s_max + extra
+    x, xd = _input(dtype, n_chan, n_samp, 7500 + n_chan + n_dm, full)
+    ref = oracle.forward(x, freqs, f_high, t_samp, ranges)[0]
+    plan = dd.Plan(freqs, f_high, t_samp, ranges, dtype)
+    got = plan.run(xd, n_samp=n_samp, segments=0)[0].cpu().numpy()
+    plan.device_status()
+    np.testing.assert_array_equal(got, ref)
+    beams = [batch.BeamSpec(freqs, f_high, t_samp, ranges, dtype, n_samp)] * 2
+    runner = batch.BatchRunner(beams, autotune=False, graph=False,
+                               tiles=[[("pattern", -1)], [("packed", -1)]])
+    for t in runner.inputs:
+        t[:, :xd.shape[1]].copy_(xd[:, :t.shape[1]])
+    for _ in range(2):
+        runner.run()
+        runner.status()
+        for i in range(2):
+            np.testing.assert_array_equal(runner.planes(i)[0].cpu().numpy(), ref)

@@ -20,6 +20,7 @@
 
 #include "dd_internal.h"
 #include "fwd_tiled.h"
+#include "host_threads.h"
 
 namespace dd {
 
@@ -180,8 +181,9 @@ bool build_pair_tables(const RangePlan& rp, int32_t n_chan, int kind, const tk::
     d = std::min<int64_t>(d, rp.n_dm - 1);
     return rp.shifts[static_cast<size_t>(d) * n_chan + c];
   };
-  std::vector<std::vector<uint32_t>> by_pat(kPatterns);
-  for (int64_t b = 0; b < n_blocks; ++b) {
+  // The blocks' tables are independent.
+  auto block = [&](int64_t b) {
+    std::vector<std::vector<uint32_t>> by_pat(kPatterns);
     const int64_t d0 = b * dm_cta;
     int32_t* bases = reinterpret_cast<int32_t*>(out.data()) + b * n_chan;
     for (int32_t c = 0; c < n_chan; ++c) bases[c] = shift(d0, c);
@@ -219,7 +221,9 @@ bool build_pair_tables(const RangePlan& rp, int32_t n_chan, int kind, const tk::
         chunk[kPairMaxWarps + w] = static_cast<unsigned char>(n - n_pairs);
       }
     }
-  }
+    return true;
+  };
+  if (!parallel_for(n_blocks, 12.0 * n_blocks * n_chan * ps.warps, block)) return false;
   *chunk_off = bases_bytes;
   *n_blocks_out = static_cast<int32_t>(n_blocks);
   return true;
@@ -580,19 +584,27 @@ dd_status build_plan(dd_plan_s* p) {
     if (rp.n_dm <= 0 || rp.n_dm > (int64_t{1} << 24))
       return fail(DD_ERR_INVALID_ARG, "range has no trial DMs or too many (max 2^24)");
     rp.shifts.resize(static_cast<size_t>(rp.n_dm) * n_chan);
-    int32_t smax = 0;
-    for (int64_t d = 0; d < rp.n_dm; ++d) {
-      double dm = rp.r.dm_lo + static_cast<double>(d) * rp.r.dm_step;
-      int32_t* row = &rp.shifts[static_cast<size_t>(d) * n_chan];
-      for (int32_t c = 0; c < n_chan; ++c) {
-        double x = delay_samples(dm, p->k[c], rp.r.bin, p->t_samp);
-        if (!(x < 1.0e9)) return fail(DD_ERR_INVALID_ARG, "shift exceeds 1e9 samples");
-        int32_t s = static_cast<int32_t>(std::floor(x + 0.5));  // round half up
-        row[c] = s;
-        smax = std::max(smax, s);
-      }
-    }
-    rp.s_max = smax;
+    // Rows of trial DMs in blocks of 64, each block's largest shift.
+    std::vector<int32_t> block_max((rp.n_dm + 63) / 64, 0);
+    if (!parallel_for(static_cast<int64_t>(block_max.size()),
+                      4.0 * static_cast<double>(rp.n_dm) * n_chan, [&](int64_t b) {
+          int32_t smax = 0;
+          for (int64_t d = 64 * b; d < std::min<int64_t>(64 * b + 64, rp.n_dm); ++d) {
+            double dm = rp.r.dm_lo + static_cast<double>(d) * rp.r.dm_step;
+            int32_t* row = &rp.shifts[static_cast<size_t>(d) * n_chan];
+            for (int32_t c = 0; c < n_chan; ++c) {
+              double x = delay_samples(dm, p->k[c], rp.r.bin, p->t_samp);
+              if (!(x < 1.0e9)) return false;
+              int32_t s = static_cast<int32_t>(std::floor(x + 0.5));  // round half up
+              row[c] = s;
+              smax = std::max(smax, s);
+            }
+          }
+          block_max[b] = smax;
+          return true;
+        }))
+      return fail(DD_ERR_INVALID_ARG, "shift exceeds 1e9 samples");
+    rp.s_max = *std::max_element(block_max.begin(), block_max.end());
     rp.gen_n_blocks = static_cast<int32_t>((rp.n_dm + kGenDmPerCta - 1) / kGenDmPerCta);
     rp.gen_span = block_span(rp, n_chan, kGenDmPerCta);
 

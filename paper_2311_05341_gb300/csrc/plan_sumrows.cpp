@@ -3,15 +3,12 @@
 // vectors of each group (its sum rows) and the moves that make one row from
 // the next.
 #include <algorithm>
-#include <atomic>
 #include <cstddef>
 #include <cstring>
-#include <new>
-#include <system_error>
-#include <thread>
 #include <vector>
 
 #include "dd_internal.h"
+#include "host_threads.h"
 #include "sumrows.h"
 
 namespace dd {
@@ -274,31 +271,11 @@ void build_sum_tables(const RangePlan& rp, int32_t n_chan, int64_t max_sample, i
   const int64_t n_blocks = (rp.n_dm + kDm - 1) / kDm;
   if (n_blocks * n_chan > (int64_t{1} << 28)) return;
 
-  // The blocks are independent: built by a few threads (those the system
-  // gives; this one takes what is left).
   std::vector<Block> blocks(n_blocks);
-  std::atomic<int64_t> next{0};
-  std::atomic<bool> ok{true};
-  auto work = [&]() {
-    try {
-      for (int64_t b = next++; b < n_blocks && ok; b = next++)
-        if (!build_block(rp, n_chan, lane_chans, f, b, &blocks[b])) ok = false;
-    } catch (const std::bad_alloc&) {
-      ok = false;
-    }
-  };
-  std::vector<std::thread> threads;
-  const int64_t want = std::min<int64_t>(
-      {n_blocks, static_cast<int64_t>(std::thread::hardware_concurrency()), 8,
-       n_blocks * n_chan / 8192 + 1});
-  try {
-    for (int64_t i = 1; i < want; ++i) threads.emplace_back(work);
-  } catch (const std::system_error&) {
-  } catch (const std::bad_alloc&) {
-  }
-  work();
-  for (auto& t : threads) t.join();
-  if (!ok) return;
+  if (!parallel_for(n_blocks, 300.0 * n_blocks * n_chan, [&](int64_t b) {
+        return build_block(rp, n_chan, lane_chans, f, b, &blocks[b]);
+      }))
+    return;
 
   size_t n_dir = 0, n_recs = 0;
   double words = 0;

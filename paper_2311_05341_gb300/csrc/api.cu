@@ -248,6 +248,11 @@ int launch_range(const dd_plan_s* p, const RangePlan& rp, const void* d_in, int6
                                   reinterpret_cast<int32_t*>(ws + tk::kStatusOffset), d_in,
                                   stride, n_out, d_out, t_begin, t_end, stream, n_out, kind,
                                   x_origin);
+  if (rp.direct.ok && dt::faster(static_cast<int32_t>(rp.n_dm), t_end - t_begin, rp.direct.kind,
+                                 rp.tile_dr))
+    return launch_forward_direct(p, rp, ws + rp.off_direct,
+                                 reinterpret_cast<int32_t*>(ws + tk::kStatusOffset), d_in, stride,
+                                 n_out, d_out, t_begin, t_end, stream);
   return rp.tile_ok ? launch_forward_tiled(p, rp, d_in, stride, n_samp, n_out, d_out, t_begin,
                                            t_end, stream)
                     : launch_forward_generic(p, rp, d_in, stride, n_samp, n_out, d_out, t_begin,

@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "dd.h"
+#include "direct.h"
 #include "fwd_tiled.h"
 #include "sumrows.h"
 
@@ -60,6 +61,9 @@ struct RangePlan {
   // kind's window alignment, a multiple of the packed kind's); 0 if none.
   int32_t alt_kind = 0;
 
+  // Direct tile of an automatic offset tile with 1 or 2 DMs per lane (direct.h).
+  DirectTables direct;
+
   // Sum-row tile of integer input (sumrows.h): from the input itself (bin 1),
   // and from the packed copies of uint8 and 4-bit input.
   SumTables sums;
@@ -70,6 +74,7 @@ struct RangePlan {
   size_t off_tile_recs = 0;     // tk::Rec or tk::PRec [tile_n_blocks][n_chan]
   size_t off_sums = 0;          // sum-row tables (sums.ok)
   size_t off_packed_sums = 0;
+  size_t off_direct = 0;        // direct tables (direct.ok)
   std::vector<unsigned char> tile_recs;  // host image of the records
 };
 
@@ -139,6 +144,10 @@ int launch_forward_tiled_with_tables(const dd_plan_s* p, const RangePlan& rp, co
                                      int32_t* err, const void* d_in, int64_t stride,
                                      int64_t n_out, void* d_out, int64_t t_begin, int64_t t_end,
                                      void* stream, bool widen_slots = true);
+// The direct tile (fwd_direct.cu), t_begin a multiple of 16.
+int launch_forward_direct(const dd_plan_s* p, const RangePlan& rp, const void* recs, int32_t* err,
+                          const void* d_in, int64_t stride, int64_t n_out, void* d_out,
+                          int64_t t_begin, int64_t t_end, void* stream);
 // The pattern kernel (fwd_pattern.cu), same arguments; output row d + 1
 // starts out_stride elements after row d (n_out for the output layout of
 // dd_run; negative for rows written in reverse order).

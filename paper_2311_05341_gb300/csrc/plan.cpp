@@ -400,12 +400,63 @@ void choose_tile(RangePlan& rp, int32_t n_chan, dd_dtype dtype) {
     if (try_tile_shape(rp, n_chan, kind, *tk::shape_for(dr))) return;
 }
 
-// choose_tile, then the sum-row tables where the tile is an integer pattern
+// Direct tile (direct.h) for an automatic offset tile of one or two DMs per
+// lane (more than 5 samples of delay a step): it reads one word per added word
+// where the offset tile reads 1.8, without a branch per DM.  Not where the
+// sums would pass its lanes (2^24) or words (2^31), or its window shared memory.
+void build_direct(RangePlan& rp, int32_t n_chan) {
+  rp.direct = DirectTables{};
+  // (Fewer than 64 trials would fill less than half of a CTA's 128.)
+  if (!rp.tile_ok || rp.tile_pattern || rp.tile_request != 0 || rp.tile_dr > 2 || rp.n_dm < 64)
+    return;
+  const int bin = rp.r.bin;
+  if (rp.tile_kind == tk::kF32 && bin > 1) return;  // its raw windows leave no such tile
+  const int kind = rp.tile_kind == tk::kF32 ? static_cast<int>(tk::kF32D) : rp.tile_kind;
+  if (kind == tk::kU8 && static_cast<int64_t>(n_chan) * 255 >= int64_t{1} << 24) return;
+  if ((kind == tk::kU8W || kind == tk::kU16) &&
+      static_cast<int64_t>(n_chan) * bin * (kind == tk::kU16 ? 65535 : 255) >= int64_t{1} << 31)
+    return;
+  const int32_t align = tk::align_samples(kind, bin);
+  const int64_t n_blocks = (rp.n_dm + dt::kDm - 1) / dt::kDm;
+  const int32_t span = block_span(rp, n_chan, dt::kDm);
+  if (span > 40000) return;
+  const int32_t lw = (dt::kWords + span + align - 1 + 15) / 16 * 16;
+  int nc = std::min(dt::kMaxNc, n_chan);
+  while (nc > 0 && dt::smem_bytes(kind, bin, nc, lw) > 227 * 1024) --nc;
+  if (nc < std::min(4, n_chan)) return;
+  rp.direct.bytes.assign(static_cast<size_t>(n_blocks) * n_chan * sizeof(dt::Rec), 0);
+  dt::Rec* recs = reinterpret_cast<dt::Rec*>(rp.direct.bytes.data());
+  const bool ok = parallel_for(n_blocks, 2.0 * n_blocks * n_chan * dt::kDm, [&](int64_t b) {
+    for (int i = 0; i < dt::kDm; ++i) {
+      const int64_t d = std::min<int64_t>(b * dt::kDm + i, rp.n_dm - 1);
+      const int32_t* row = &rp.shifts[static_cast<size_t>(d) * n_chan];
+      for (int32_t c = 0; c < n_chan; ++c) {
+        dt::Rec& r = recs[b * n_chan + c];
+        if (i == 0) r.base = row[c];
+        if (row[c] < r.base) return false;
+        r.off[i] = static_cast<uint16_t>(row[c] - r.base + r.base % align);
+      }
+    }
+    return true;
+  });
+  if (!ok) {
+    rp.direct = DirectTables{};
+    return;
+  }
+  rp.direct.kind = kind;
+  rp.direct.n_blocks = static_cast<int32_t>(n_blocks);
+  rp.direct.nc = nc;
+  rp.direct.lw = lw;
+  rp.direct.ok = true;
+}
+
+// choose_tile, then the direct tables, then the sum-row tables where the tile is an integer pattern
 // tile of the automatic shape (time tiles of 32 x 23 words): from the input
 // itself at bin 1; from the packed copy of uint8 (any bin of its packed tile)
 // and 4-bit input, which is faster where the caller gives scratch for it.
 void choose_kernels(RangePlan& rp, int32_t n_chan, dd_dtype dtype) {
   choose_tile(rp, n_chan, dtype);
+  build_direct(rp, n_chan);
   rp.sums = SumTables{};
   rp.packed_sums = SumTables{};
   if (!rp.tile_ok || !rp.tile_pattern || rp.shape_request >= 0 || dtype == DD_F32 ||
@@ -469,6 +520,11 @@ void layout_workspace(dd_plan_s* p) {
       rp.off_tile_recs = ws;
       ws += rp.tile_recs.size();
     }
+    if (rp.direct.ok) {
+      ws = align_up(ws, 256);
+      rp.off_direct = ws;
+      ws += rp.direct.bytes.size();
+    }
     // Sum-row tables: room for both sets, a power of two each, so that the
     // workspace's size depends on the plan's shape and not on which window
     // formats its dtype has.
@@ -507,6 +563,9 @@ void layout_workspace(dd_plan_s* p) {
                 rp.shifts.size() * sizeof(int32_t));
     if (rp.tile_ok)
       std::memcpy(p->host_ws.data() + rp.off_tile_recs, rp.tile_recs.data(), rp.tile_recs.size());
+    if (rp.direct.ok)
+      std::memcpy(p->host_ws.data() + rp.off_direct, rp.direct.bytes.data(),
+                  rp.direct.bytes.size());
     if (rp.sums.ok)
       std::memcpy(p->host_ws.data() + rp.off_sums, rp.sums.bytes.data(), rp.sums.bytes.size());
     if (rp.packed_sums.ok)

@@ -1,0 +1,55 @@
+// tmem.cuh -- the high bytes of 16-bit accumulator lanes in tensor memory.
+//
+// Two samples share a 32-bit accumulator word.  Before the lanes can overflow,
+// a flush moves each lane's high byte to the word's column in tensor memory
+// (16-bit sums of high bytes, below 2^16 while the total stays below 2^24) and
+// keeps the low byte: 255 x 256 more fits the lane.  Partial sums so never
+// leave the SM.  A CTA that allocates all 512 columns must be the only one on
+// its SM (its shared memory sees to that).
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+namespace dd {
+namespace tmem {
+
+// By one warp; the address comes back in shared memory.
+__device__ __forceinline__ void alloc(uint32_t dst) {
+  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(dst)
+               : "memory");
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void dealloc(uint32_t addr) {
+  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(addr) : "memory");
+}
+__device__ __forceinline__ void fence_before() {
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+}
+__device__ __forceinline__ void fence_after() {
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+}
+// Columns of warp w: its quarter of the lanes (32 (w % 4) + t for thread t) and
+// `cols` columns for each of the warps that share the quarter.
+__device__ __forceinline__ uint32_t warp_columns(uint32_t base, int w, int cols) {
+  return base + (static_cast<uint32_t>(32 * (w & 3)) << 16) + static_cast<uint32_t>(cols * (w >> 2));
+}
+__device__ __forceinline__ void load4(uint32_t addr, uint32_t (&v)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+               : "r"(addr)
+               : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void store4(uint32_t addr, const uint32_t (&v)[4]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr),
+               "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3])
+               : "memory");
+}
+__device__ __forceinline__ void wait_stores() {
+  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+
+}  // namespace tmem
+}  // namespace dd

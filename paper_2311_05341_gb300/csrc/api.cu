@@ -238,7 +238,15 @@ int launch_range(const dd_plan_s* p, const RangePlan& rp, const void* d_in, int6
                  void* stream, int kind = 0, int64_t x_origin = 0) {
   unsigned char* ws = static_cast<unsigned char*>(p->d_ws);
   const SumTables& sums = kind > 0 ? rp.packed_sums : rp.sums;
-  if (sums.ok)
+  // Bin 2 from the input: the pattern tile's units (64 DMs x 736 outputs) are
+  // half as large and 0.8 of the time each, which tells in less than a wave.
+  auto load = [](int64_t dms, int64_t per_dms, int64_t outs) {
+    const int64_t ctas = (dms + per_dms - 1) / per_dms * ((outs + 735) / 736);
+    return ctas < 152 ? 1.0 : static_cast<double>(ctas) / 152;
+  };
+  const bool small = sums.src == sr::kBytes2 && 1.25 * load(rp.n_dm, 128, t_end - t_begin) >
+                                                    load(rp.n_dm, 64, t_end - t_begin);
+  if (sums.ok && !small)
     return launch_forward_sum_rows(p, rp, sums,
                                    ws + (kind > 0 ? rp.off_packed_sums : rp.off_sums),
                                    reinterpret_cast<int32_t*>(ws + tk::kStatusOffset), d_in,

@@ -162,13 +162,14 @@ int launch_forward_pattern(const dd_plan_s* p, const RangePlan& rp, const void* 
                            bool widen_slots = true);
 // The sum-row kernel (fwd_sumrows.cu) on the rows sums.src names (the input,
 // or words of its packed copy); stride in their samples, x_origin and the
-// times as launch_forward_pattern.
+// times as launch_forward_pattern (t_begin a multiple of 736 or, in words, 368
+// samples; from a packed copy 1472).
 int launch_forward_sum_rows(const dd_plan_s* p, const RangePlan& rp, const SumTables& sums,
                             const void* tables,
                             int32_t* err, const void* d_rows, int64_t stride, void* d_out,
                             int64_t t_begin, int64_t t_end, void* stream, int64_t out_stride,
                             int64_t x_origin);
-// Its launch parameters (x_origin and tile0 zero), the 368-word halves of time
+// Its launch parameters (x_origin and half0 zero), the 368-word halves of time
 // tiles that outputs [t_begin, t_end) take, and the persistent kernel of one
 // window format (sr::Src).
 sr::Params sum_row_params(const dd_plan_s* p, const RangePlan& rp, const SumTables& sums,

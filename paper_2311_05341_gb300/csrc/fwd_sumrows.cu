@@ -177,9 +177,9 @@ struct Lane;
 
 template <>
 struct Lane<kPairs> {
-  static constexpr int kN = 5, kLoads = 6, kDepth = 2;
+  static constexpr int kN = 5, kStep = 5, kLoads = 6, kDepth = 2;
   uint32_t base;  // shared address of the lane's first word at offset 0
-  __device__ Lane(uint32_t raw, int k) : base(raw + 4u * k) {}
+  __device__ Lane(uint32_t raw, int k, int) : base(raw + 4u * k) {}
   __device__ void load(uint32_t (&x)[kLoads], uint32_t offset) const {
     const uint32_t a = base + 4u * (offset & 0xffffu);
 #pragma unroll
@@ -232,9 +232,9 @@ struct SplitPairs {
 
 template <>
 struct Lane<kBytes> : SplitPairs {
-  static constexpr int kN = 4, kLoads = 4, kDepth = 3;
+  static constexpr int kN = 4, kStep = 4, kLoads = 4, kDepth = 3;
   uint32_t base;
-  __device__ Lane(uint32_t raw, int k) : base(raw + k) {}  // k a multiple of 4
+  __device__ Lane(uint32_t raw, int k, int) : base(raw + k) {}  // k a multiple of 4
   __device__ void load_first(uint32_t (&x)[kLoads], uint32_t offset) const { load(x, offset); }
   __device__ void load(uint32_t (&x)[kLoads], uint32_t offset) const {
     const uint32_t a = base + (offset & 0xfffcu);
@@ -268,10 +268,10 @@ struct Lane<kBytes> : SplitPairs {
 
 template <>
 struct Lane<kNibbles> : SplitPairs {
-  static constexpr int kN = 4, kLoads = 4, kDepth = 3;
+  static constexpr int kN = 4, kStep = 4, kLoads = 4, kDepth = 3;
   uint32_t raw;
   int k;
-  __device__ Lane(uint32_t raw_, int k_) : raw(raw_), k(k_) {}
+  __device__ Lane(uint32_t raw_, int k_, int) : raw(raw_), k(k_) {}
   __device__ void load_first(uint32_t (&x)[kLoads], uint32_t offset) const { load(x, offset); }
   __device__ void load(uint32_t (&x)[kLoads], uint32_t offset) const {
     const uint32_t a = raw + (((offset & 0xffffu) + k) >> 3) * 4u;
@@ -305,11 +305,13 @@ struct Lane<kNibbles> : SplitPairs {
   }
 };
 
+// uint16: four words in a row.  (Two pieces of two words, 64 apart, would load
+// without bank conflicts but with four loads for three: 20.7 against 19.2 ms.)
 template <>
 struct Lane<kHalves> {
-  static constexpr int kN = 4, kLoads = 3, kDepth = 3;
+  static constexpr int kN = 4, kStep = 4, kLoads = 3, kDepth = 3;
   uint32_t base;
-  __device__ Lane(uint32_t raw, int k) : base(raw + 2u * k) {}  // k a multiple of 4
+  __device__ Lane(uint32_t raw, int k, int) : base(raw + 2u * k) {}  // k a multiple of 4
   __device__ void load_first(uint32_t (&x)[kLoads], uint32_t offset) const { load(x, offset); }
   __device__ void load(uint32_t (&x)[kLoads], uint32_t offset) const {
     const uint32_t a = base + 2u * (offset & 0xfffeu);
@@ -340,8 +342,60 @@ struct Lane<kHalves> {
   }
 };
 
+// uint8 decimated by 2 from the input: two pieces of two words, 64 words apart
+// (the lanes of a load take consecutive 32-bit words): s[0], s[1] the first
+// piece's two decimated samples and those 368 later as 16-bit pairs, s[2], s[3]
+// the second's.
+template <>
+struct Lane<kBytes2> {
+  static constexpr int kN = 4, kStep = 2, kLoads = 8, kDepth = 2;
+  uint32_t base;
+  uint32_t d;  // words from the first piece to the second
+  __device__ Lane(uint32_t raw, int k, int rs) : base(raw + 2u * k), d(min(64, rs - 2 - k)) {}
+  __device__ void load_first(uint32_t (&x)[kLoads], uint32_t offset) const { load(x, offset); }
+  __device__ void load(uint32_t (&x)[kLoads], uint32_t offset) const {
+    const uint32_t a = base + 2u * (offset & 0xfffeu), b = a + 2u * d;
+    x[0] = lds(a);
+    x[1] = lds(a + 4);
+    x[2] = lds(a + 2 * kWords);
+    x[3] = lds(a + 2 * kWords + 4);
+    x[4] = lds(b);
+    x[5] = lds(b + 4);
+    x[6] = lds(b + 2 * kWords);
+    x[7] = lds(b + 2 * kWords + 4);
+  }
+  // Two decimated samples of four bytes, as a 16-bit pair.
+  __device__ static uint32_t decimate(uint32_t y) {
+    return (y & 0x00ff00ffu) + __byte_perm(y, 0u, 0x4341);
+  }
+  __device__ void first(uint32_t (&s)[kN], const uint32_t (&x)[kLoads], uint32_t offset) const {
+    const uint32_t sh = 16u * (offset & 1u);
+#pragma unroll
+    for (int h = 0; h < 4; ++h) s[h] += decimate(__funnelshift_r(x[2 * h], x[2 * h + 1], sh));
+  }
+  __device__ void move(uint32_t (&s)[kN], const uint32_t (&x)[kLoads], uint32_t offset,
+                       uint32_t sign) const {
+    const uint32_t sh = 16u * (offset & 1u);
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const uint32_t p = decimate(__funnelshift_r(x[2 * h], x[2 * h + 1], sh));
+      const uint32_t q = decimate(x[2 * h + 1] >> sh);
+      s[h] += (__byte_perm(p, q, 0x5432) - p) * sign;
+    }
+  }
+  __device__ void store(uint32_t a, const uint32_t (&s)[kN], uint32_t on) const {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %6, 0;\n\t"
+        "@p st.shared.v2.u32 [%0], {%2, %3};\n\t@p st.shared.v2.u32 [%1], {%4, %5};\n\t}" ::"r"(a),
+        "r"(a + 4u * d), "r"(__byte_perm(s[0], s[1], 0x5410)),
+        "r"(__byte_perm(s[0], s[1], 0x7632)), "r"(__byte_perm(s[2], s[3], 0x5410)),
+        "r"(__byte_perm(s[2], s[3], 0x7632)), "r"(on)
+        : "memory");
+  }
+};
+
 // One group's rows, by warp bw of a building warpgroup: chunks of 32 kN row
-// words, kN consecutive ones per lane.  Lanes past the row repeat its last
+// words, lane l's first one kStep l words on; lanes past the row repeat its last
 // words.  Loads run a channel pair, then kDepth moves ahead of the sums.
 template <int SRC>
 __device__ __forceinline__ void build_rows(const unsigned char* rec, uint32_t raw, uint32_t rows,
@@ -351,8 +405,8 @@ __device__ __forceinline__ void build_rows(const unsigned char* rec, uint32_t ra
   static_assert(kN == format(SRC).build && kDepth <= kStepPad / 2, "planner's lane width");
   const RecHead h = *reinterpret_cast<const RecHead*>(rec);
   for (int chunk = bw; chunk * (32 * kN) < h.rs; chunk += kBuildWarps) {
-    const int k0 = min(chunk * (32 * kN) + kN * lane, h.rs - kN);
-    const L win(raw, k0);
+    const int k0 = min(chunk * (32 * kN) + L::kStep * lane, h.rs - L::kStep);
+    const L win(raw, k0, h.rs);
     const uint32_t rs4 = 4u * h.rs;
     uint32_t dst = rows + 4u * k0;
     uint32_t s[kN];
@@ -389,7 +443,7 @@ __device__ __forceinline__ void build_rows(const unsigned char* rec, uint32_t ra
         win.first(s, a0, oa);
       }
     }
-    L::store(dst, s, 1u);
+    win.store(dst, s, 1u);
     dst += rs4;
     const uint32_t* steps = reinterpret_cast<const uint32_t*>(rec + rec_steps_off(h.k));
     uint32_t x[kDepth][L::kLoads], st[kDepth], nx[kDepth];
@@ -409,7 +463,7 @@ __device__ __forceinline__ void build_rows(const unsigned char* rec, uint32_t ra
         win.load(x[e], nx[e]);
         st[e] = nx[e];
         nx[e] = steps[kDepth + e];
-        L::store(dst, s, on);
+        win.store(dst, s, on);
         dst += on ? rs4 : 0u;
       }
     }
@@ -615,12 +669,15 @@ __device__ __forceinline__ void init_barriers(Ctl* ctl) {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 
-// First output sample of half `half` of the time tiles (736 x 2 samples in
-// 16-bit lanes, 736 in words): a half holds 368 words.
+// First output sample of half half0 + i (368 words) of the time axis.  Halves
+// of packed-copy tiles (736 words, 1472 samples; half0 even) interleave; the
+// others are in order.  (32-bit unsigned i: a signed 64-bit division here cost
+// the adders' registers, 12 % of the kernel.)
 template <int SRC>
-__device__ __forceinline__ int64_t half_origin(int64_t tile0, int64_t half) {
-  if constexpr (SRC == kPairs) return (tile0 + half / 2) * (2 * kPairWords) + (half % 2) * kWords;
-  else return (2 * tile0 + half) * (lanes16(SRC) ? 2 * kWords : kWords);
+__device__ __forceinline__ int64_t half_origin(int64_t half0, uint32_t i) {
+  if constexpr (SRC == kPairs)
+    return half0 * kPairWords + static_cast<int64_t>(i / 2) * (2 * kPairWords) + (i % 2) * kWords;
+  else return (half0 + i) * (lanes16(SRC) ? 2 * kWords : kWords);
 }
 
 template <int SRC>
@@ -635,8 +692,8 @@ __global__ void __launch_bounds__(kThreads, 1) sum_row_kernel(const __grid_const
   }
   __syncthreads();
   if constexpr (LANES16) tmem_fence_after();
-  const int blk = blockIdx.x % p.n_blocks;
-  const int64_t w0 = half_origin<SRC>(p.tile0, blockIdx.x / p.n_blocks);
+  const int blk = blockIdx.x % static_cast<uint32_t>(p.n_blocks);
+  const int64_t w0 = half_origin<SRC>(p.half0, blockIdx.x / static_cast<uint32_t>(p.n_blocks));
   const int32_t* first = reinterpret_cast<const int32_t*>(p.tables);
   const int g0 = first[blk], n_groups = first[blk + 1] - g0;
   // 256 x 208 + 256 x 48 registers: the 512 x 128 of the launch.
@@ -710,7 +767,7 @@ __global__ void __launch_bounds__(kThreads, 1) sum_row_batch_kernel(const BatchA
     const tk::BatchItem item = b.items[bc->item];
     const int32_t* first = reinterpret_cast<const int32_t*>(bc->p.tables);
     *blk = item.blk;
-    *w0 = half_origin<SRC>(bc->p.tile0, item.tile);
+    *w0 = half_origin<SRC>(bc->p.half0, static_cast<uint32_t>(item.tile));
     *g0 = first[item.blk];
     *n_groups = first[item.blk + 1] - *g0;
   };
@@ -768,7 +825,9 @@ sr::Params sum_row_params(const dd_plan_s* p, const RangePlan& rp, const SumTabl
                           void* d_out, int64_t t_end, int64_t out_stride) {
   sr::Params prm{};
   prm.x = d_rows;
-  prm.stride = stride;
+  // In staged samples: the decimated ones of a row (a partial one at its end
+  // holds no output's sample).
+  prm.stride = sums.src == sr::kBytes2 ? stride / 2 : stride;
   prm.n_chan = p->n_chan;
   prm.n_dm = static_cast<int32_t>(rp.n_dm);
   prm.n_blocks = sums.n_blocks;
@@ -785,13 +844,13 @@ sr::Params sum_row_params(const dd_plan_s* p, const RangePlan& rp, const SumTabl
 }
 
 int64_t sum_row_halves(int src, int64_t t_begin, int64_t t_end) {
+  const int64_t half = sr::kWords * (sr::lanes16(src) ? 2 : 1);
+  if (src != sr::kPairs) return (t_end + half - 1) / half - t_begin / half;
   // A half of a packed-copy tile holds its first 368 samples and those 736
-  // later, so the last tile's second half only counts where the tile has more
-  // than 368 outputs; the others' halves are in order.
-  const int64_t half = sr::kWords * (sr::lanes16(src) ? 2 : 1), ts = 2 * half;
-  const int64_t whole = t_end / ts - t_begin / ts, rest = t_end % ts;
-  const int64_t second = src == sr::kPairs ? sr::kWords : half;
-  return 2 * whole + (rest > second ? 2 : rest > 0 ? 1 : 0);
+  // later: the last tile's second half only counts where the tile has more
+  // than 368 outputs.
+  const int64_t ts = 2 * half, whole = t_end / ts - t_begin / ts, rest = t_end % ts;
+  return 2 * whole + (rest > sr::kWords ? 2 : rest > 0 ? 1 : 0);
 }
 
 int launch_sum_row_batch(int src, const sr::BatchArgs& args, int32_t grid, void* stream) {
@@ -801,6 +860,7 @@ int launch_sum_row_batch(int src, const sr::BatchArgs& args, int32_t grid, void*
     case sr::kBytes: return sr::launch_batch<sr::kBytes>(args, grid, st);
     case sr::kNibbles: return sr::launch_batch<sr::kNibbles>(args, grid, st);
     case sr::kHalves: return sr::launch_batch<sr::kHalves>(args, grid, st);
+    case sr::kBytes2: return sr::launch_batch<sr::kBytes2>(args, grid, st);
   }
   return static_cast<int>(cudaErrorInvalidValue);
 }
@@ -810,14 +870,14 @@ int launch_forward_sum_rows(const dd_plan_s* p, const RangePlan& rp, const SumTa
                             int64_t t_begin, int64_t t_end, void* stream, int64_t out_stride,
                             int64_t x_origin) {
   const int src = sums.src;
-  const int64_t ts = 2 * sr::kWords * (sr::lanes16(src) ? 2 : 1);  // pattern time tiles
-  if (x_origin < 0 || x_origin % sr::format(src).align != 0 || t_begin % ts != 0 || t_begin < 0 ||
-      t_end <= t_begin)
+  const int64_t half = sr::kWords * (sr::lanes16(src) ? 2 : 1);
+  if (x_origin < 0 || x_origin % sr::format(src).align != 0 || t_begin < 0 ||
+      t_begin % (src == sr::kPairs ? 2 * half : half) != 0 || t_end <= t_begin)
     return static_cast<int>(cudaErrorInvalidValue);
   sr::Params prm =
       sum_row_params(p, rp, sums, tables, err, d_rows, stride, d_out, t_end, out_stride);
   prm.x_origin = x_origin;
-  prm.tile0 = t_begin / ts;
+  prm.half0 = t_begin / half;
   const int64_t halves = sum_row_halves(src, t_begin, t_end);
   const int64_t grid = halves * prm.n_blocks;
   if (grid <= 0 || grid > 0x7fffffffLL) return static_cast<int>(cudaErrorInvalidConfiguration);
@@ -827,6 +887,7 @@ int launch_forward_sum_rows(const dd_plan_s* p, const RangePlan& rp, const SumTa
     case sr::kBytes: return sr::launch<sr::kBytes>(prm, grid, st);
     case sr::kNibbles: return sr::launch<sr::kNibbles>(prm, grid, st);
     case sr::kHalves: return sr::launch<sr::kHalves>(prm, grid, st);
+    case sr::kBytes2: return sr::launch<sr::kBytes2>(prm, grid, st);
   }
   return static_cast<int>(cudaErrorInvalidValue);
 }

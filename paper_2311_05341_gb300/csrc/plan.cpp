@@ -452,7 +452,7 @@ void build_direct(RangePlan& rp, int32_t n_chan) {
 
 // choose_tile, then the direct tables, then the sum-row tables where the tile is an integer pattern
 // tile of the automatic shape (time tiles of 32 x 23 words): from the input
-// itself at bin 1; from the packed copy of uint8 (any bin of its packed tile)
+// itself at bin 1 (uint8 also at bin 2); from the packed copy of uint8 (any bin of its packed tile)
 // and 4-bit input, which is faster where the caller gives scratch for it.
 void choose_kernels(RangePlan& rp, int32_t n_chan, dd_dtype dtype) {
   choose_tile(rp, n_chan, dtype);
@@ -469,6 +469,8 @@ void choose_kernels(RangePlan& rp, int32_t n_chan, dd_dtype dtype) {
                      : dtype == DD_U4 ? sr::kNibbles
                                       : sr::kBytes,
                      &rp.sums);
+  else if (rp.r.bin == 2 && rp.tile_kind == tk::kU8W)
+    build_sum_tables(rp, n_chan, 2 * top, sr::kBytes2, &rp.sums);
   if (copy_kind(rp, true) == tk::kU8P)
     build_sum_tables(rp, n_chan, top * rp.r.bin, sr::kPairs, &rp.packed_sums);
 }

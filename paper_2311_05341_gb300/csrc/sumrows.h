@@ -54,8 +54,9 @@ constexpr int kMaxRec = 16 + kMaxK * 2 + (kMaxSteps + kStepPad) * 4 + kDm * 2 + 
 // 736 apart, in 16-bit lanes), for decimated uint8.  kBytes, kNibbles: the
 // uint8 or 4-bit input itself; a row word pairs samples 368 apart, so a CTA's
 // 736 outputs and its staged window are contiguous.  kHalves: the uint16
-// input, one sample per 32-bit row word.
-enum Src : int { kPairs = 0, kBytes = 1, kNibbles = 2, kHalves = 3 };
+// input, one sample per 32-bit row word.  kBytes2: the uint8 input decimated by
+// 2 as it is read, row words as kBytes (staged samples are the decimated ones).
+enum Src : int { kPairs = 0, kBytes = 1, kNibbles = 2, kHalves = 3, kBytes2 = 4 };
 
 struct Format {
   int bits;        // per staged sample (kPairs: per word)
@@ -77,7 +78,8 @@ DD_HOST_DEVICE constexpr Format format(int src) {
   return src == kPairs      ? Format{32, 16, 5, 1, 29696, 11392, 110, 155}
          : src == kBytes    ? Format{8, 16, 4, kWords + 8, 17408, 14464, 190, 145}
          : src == kNibbles  ? Format{4, 32, 4, kWords + 16, 17408, 14464, 195, 165}
-                            : Format{16, 16, 4, 4, 17408, 14464, 380, 130};
+         : src == kHalves   ? Format{16, 16, 4, 4, 17408, 14464, 380, 130}
+                            : Format{16, 16, 4, kWords + 4, 29696, 11392, 300, 200};
 }
 // Output samples of a CTA's words, and of the pattern time tile holding them.
 DD_HOST_DEVICE constexpr int pair_dist(int src) { return src == kPairs ? kPairWords : kWords; }
@@ -135,7 +137,8 @@ DD_HOST_DEVICE constexpr size_t row_off(int src) {
 DD_HOST_DEVICE constexpr size_t smem_bytes(int src) {
   return row_off(src) + kSlots * static_cast<size_t>(format(src).row_words) * 4;
 }
-static_assert(smem_bytes(kPairs) <= 227 * 1024 && smem_bytes(kBytes) <= 227 * 1024,
+static_assert(smem_bytes(kPairs) <= 227 * 1024 && smem_bytes(kBytes) <= 227 * 1024 &&
+                  smem_bytes(kBytes2) <= 227 * 1024,
               "sum-row tile exceeds shared memory");
 
 struct Params {
@@ -148,7 +151,7 @@ struct Params {
   const unsigned char* tables;
   int32_t off_dir;       // byte offsets of the directory and the window starts
   int32_t off_start;
-  int64_t tile0;         // first pattern time tile of the launch
+  int64_t half0;         // first half of the launch (half_origin)
   int64_t t_end;         // outputs t >= t_end are not written
   int64_t out_stride;    // elements from output row d to row d + 1
   int32_t* out;

@@ -165,3 +165,38 @@ def test_sum_row_tile_from_the_input(dtype, n_chan, n_dm, slope, extra, full):
         runner.status()
         for i in range(2):
             np.testing.assert_array_equal(runner.planes(i)[0].cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("n_chan,n_dm,slope,extra,full", [
+    (513, 200, 0.2, 1841, True), (1000, 129, 0.15, 735, False), (2047, 256, 0.9, 737, True),
+    (600, 1, 0.5, 1, False)])
+def test_sum_row_tile_decimates_the_input_by_two(n_chan, n_dm, slope, extra, full):
+    """Bin 2 from the input: alone, as a window, through the segmented host
+    pipeline (segments start at multiples of 736 outputs) and in a batch."""
+    from paper_2311_05341_gb300 import batch
+    f_high, t_samp = 1500.0, 64e-6
+    freqs = channel_freqs(f_high, 300.0, n_chan)
+    step = slope * 2 * t_samp / oracle.delay_coeff(freqs[-1], f_high)
+    ranges = [(0.0, n_dm * step, step, 2)]
+    s_max = oracle.extent(freqs, f_high, t_samp, ranges[0], 10 ** 9)[0]
+    n_samp = 2 * (s_max + extra) + 1
+    x, xd = _input("u8", n_chan, n_samp, 7700 + n_chan, full)
+    ref = oracle.forward(x, freqs, f_high, t_samp, ranges)[0]
+    plan = dd.Plan(freqs, f_high, t_samp, ranges, "u8")
+    got = plan.run(xd, n_samp=n_samp)[0].cpu().numpy()
+    plan.device_status()
+    np.testing.assert_array_equal(got, ref)
+    keep = max(1, extra // 2)
+    got = plan.run_window(xd, [keep], n_samp=n_samp)[0].cpu().numpy()
+    np.testing.assert_array_equal(got, ref[:, :keep])
+    h_in, d_out = xd.cpu().pin_memory(), plan.empty_output(n_samp)
+    h_out = torch.full(d_out.shape, -1, dtype=d_out.dtype).pin_memory()
+    plan.run_host(h_in, h_out, torch.zeros_like(xd), d_out, n_samp=n_samp)
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(plan.split(h_out, n_samp)[0].numpy(), ref)
+    runner = batch.BatchRunner([batch.BeamSpec(freqs, f_high, t_samp, ranges, "u8", n_samp)],
+                               autotune=False, graph=False)
+    runner.inputs[0][:, :xd.shape[1]].copy_(xd[:, :runner.inputs[0].shape[1]])
+    runner.run()
+    runner.status()
+    np.testing.assert_array_equal(runner.planes(0)[0].cpu().numpy(), ref)

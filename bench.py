@@ -46,9 +46,10 @@ def _measured_hbm_gbs(default=6800.0):
 HBM_GBS = _measured_hbm_gbs()
 # dram__bytes_read.sum + dram__bytes_write.sum of the transform launches the
 # roofline times (ncu), keyed by workload, raw samples, tiles, input mode and
-# segments; valid only for the kernel build it was taken on
-# (profiles/fwd_pattern_u8_8192ch.md).
-TRAFFIC = {("paper_u8", 262144, (0x104,), "packed ring", 8): 18.29e9 + 13.42e9}
+# segments; valid only for the kernel build it was taken on.  None is held for
+# the sum-row tile (the pattern tile's 31.7 GB of widenings and re-reads on
+# paper_u8 do not apply to it).
+TRAFFIC = {}
 UNIT = "DM*samples/s"
 
 
@@ -321,6 +322,9 @@ def run_ours(args):
     roofline = {
         "bound": "alu", "achieved": sample_adds_per_s / 1e12, "peak": peak_adds / 1e12,
         "unit": "Tadd/s", "frac": sample_adds_per_s / peak_adds,
+        # The direct sum's additions: a tile that adds sums of channels shared by
+        # trial DMs takes fewer, so the fraction may pass 1.
+        "counted": "direct sum: one add per (trial DM, output sample, channel)",
         "traffic": traffic,
         "kernel_ms": kern * 1e3,
         "timed": ("the whole step: %d transform launches on two streams with the packing "

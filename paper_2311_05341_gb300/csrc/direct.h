@@ -1,5 +1,5 @@
 // direct.h -- geometry, tables and launch parameters of the direct tile
-// (fwd_direct.cu) for steep plans: more than 7 samples of delay between
+// (fwd_direct.cu) for steep plans: more than 5 samples of delay between
 // consecutive trial DMs, where the words one trial loads serve no other.
 //
 // A CTA takes 128 trial DMs x 368 window words of one channel after another:

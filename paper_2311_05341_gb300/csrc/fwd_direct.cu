@@ -156,14 +156,14 @@ __global__ void __launch_bounds__(32 * kWarps, 1) direct_kernel(const __grid_con
 #pragma unroll
         for (int q = 0; q < kPairs * kAcc; q += 4) {
           uint32_t v[4] = {};
-          if (flushed) tmem::load4(col + q, v);
+          if (flushed) tmem::load(col + q, v);
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
             uint32_t& a = acc[(q + e) / kAcc][(q + e) % kAcc];
             v[e] += __byte_perm(a, 0u, 0x4341);
             a &= 0x00ff00ffu;
           }
-          tmem::store4(col + q, v);
+          tmem::store(col + q, v);
         }
         tmem::wait_stores();
         flushed = true;
@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(32 * kWarps, 1) direct_kernel(const __grid_con
       uint32_t v[4] = {};
       if (kLanes16 && flushed) {
         __syncwarp();
-        tmem::load4(col + q, v);
+        tmem::load(col + q, v);
       }
 #pragma unroll
       for (int e = 0; e < 4; ++e) {

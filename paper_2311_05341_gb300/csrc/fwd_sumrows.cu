@@ -43,6 +43,7 @@
 #include "dd_internal.h"
 #include "sumrows.h"
 #include "tile_common.cuh"
+#include "tmem.cuh"
 
 namespace dd {
 namespace sr {
@@ -102,42 +103,6 @@ __device__ __forceinline__ void mbar_inval(uint32_t bar) {
   asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-// Tensor memory: all 512 columns (the tile's shared memory admits one CTA per
-// SM); thread t of a warp reaches lane 32 (warp % 4) + t.
-__device__ __forceinline__ void tmem_alloc(uint32_t dst) {
-  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(dst)
-               : "memory");
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t addr) {
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(addr) : "memory");
-}
-__device__ __forceinline__ void tmem_load8(uint32_t addr, uint32_t (&v)[8]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]),
-                 "=r"(v[6]), "=r"(v[7])
-               : "r"(addr)
-               : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_store8(uint32_t addr, const uint32_t (&v)[8]) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(
-                   addr),
-               "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]),
-               "r"(v[7])
-               : "memory");
-}
-__device__ __forceinline__ void tmem_wait_stores() {
-  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ void tmem_fence_before() {
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_fence_after() {
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-}
-
 constexpr int kDmPairs = kDmWarp / 2;
 static_assert(kDmPairs * kAcc % 8 == 0, "tensor memory moves 8 words at a time");
 
@@ -149,16 +114,16 @@ __device__ __forceinline__ void flush_lanes(uint32_t col, uint32_t (&acc)[kDmPai
 #pragma unroll
   for (int q = 0; q < kDmPairs * kAcc; q += 8) {
     uint32_t v[8] = {};
-    if (!first) tmem_load8(col + q, v);
+    if (!first) tmem::load(col + q, v);
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       uint32_t& a = acc[(q + e) / kAcc][(q + e) % kAcc];
       v[e] += __byte_perm(a, 0u, 0x4341);
       a &= 0x00ff00ffu;
     }
-    tmem_store8(col + q, v);
+    tmem::store(col + q, v);
   }
-  tmem_wait_stores();
+  tmem::wait_stores();
 }
 
 __device__ __forceinline__ uint32_t lds(uint32_t a) {
@@ -560,8 +525,7 @@ __device__ __forceinline__ void add_and_store(const Params& p, unsigned char* sm
                                               int blk, int64_t w0, int g0, int n_groups) {
   constexpr bool LANES16 = lanes16(SRC);
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t col =
-      LANES16 ? ctl->tmem + (static_cast<uint32_t>(32 * (w & 3)) << 16) + 256u * (w >> 2) : 0u;
+  const uint32_t col = LANES16 ? tmem::warp_columns(ctl->tmem, w, 256) : 0u;
   uint32_t acc[kDmPairs][kAcc];
 #pragma unroll
   for (int i = 0; i < kDmPairs; ++i)
@@ -644,7 +608,7 @@ __device__ __forceinline__ void add_and_store(const Params& p, unsigned char* sm
     uint32_t v[8] = {};
     if (LANES16 && flushed) {
       __syncwarp();
-      tmem_load8(col + q, v);
+      tmem::load(col + q, v);
     }
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
@@ -687,11 +651,11 @@ __global__ void __launch_bounds__(kThreads, 1) sum_row_kernel(const __grid_const
   Ctl* ctl = reinterpret_cast<Ctl*>(smem);
   if (threadIdx.x == 0) init_barriers<SRC>(ctl);
   if constexpr (LANES16) {
-    if (threadIdx.x < 32) tmem_alloc(smem_u32(&ctl->tmem));
-    tmem_fence_before();
+    if (threadIdx.x < 32) tmem::alloc(smem_u32(&ctl->tmem));
+    tmem::fence_before();
   }
   __syncthreads();
-  if constexpr (LANES16) tmem_fence_after();
+  if constexpr (LANES16) tmem::fence_after();
   const int blk = blockIdx.x % static_cast<uint32_t>(p.n_blocks);
   const int64_t w0 = half_origin<SRC>(p.half0, blockIdx.x / static_cast<uint32_t>(p.n_blocks));
   const int32_t* first = reinterpret_cast<const int32_t*>(p.tables);
@@ -704,13 +668,13 @@ __global__ void __launch_bounds__(kThreads, 1) sum_row_kernel(const __grid_const
     asm volatile("setmaxnreg.inc.sync.aligned.u32 208;");
     add_and_store<SRC>(p, smem, ctl, blk, w0, g0, n_groups);
   }
-  if constexpr (LANES16) tmem_fence_before();
+  if constexpr (LANES16) tmem::fence_before();
   __syncthreads();
   if (ctl->abort && threadIdx.x == 0) drain_copies(ctl);
   if constexpr (LANES16) {
-    tmem_fence_after();
+    tmem::fence_after();
     __syncwarp();
-    if (threadIdx.x < 32) tmem_dealloc(ctl->tmem);
+    if (threadIdx.x < 32) tmem::dealloc(ctl->tmem);
   }
 }
 
@@ -736,8 +700,8 @@ __global__ void __launch_bounds__(kThreads, 1) sum_row_batch_kernel(const BatchA
   BatchCtl* bc = reinterpret_cast<BatchCtl*>(smem);
   Ctl* ctl = &bc->ctl;
   if constexpr (LANES16) {
-    if (threadIdx.x < 32) tmem_alloc(smem_u32(&ctl->tmem));
-    tmem_fence_before();
+    if (threadIdx.x < 32) tmem::alloc(smem_u32(&ctl->tmem));
+    tmem::fence_before();
   }
   // The next item, or false: none is left or the last one was given up.
   bool fresh = true;
@@ -783,18 +747,18 @@ __global__ void __launch_bounds__(kThreads, 1) sum_row_batch_kernel(const BatchA
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 208;");
     while (next_item()) {
-      if constexpr (LANES16) tmem_fence_after();
+      if constexpr (LANES16) tmem::fence_after();
       unit(&blk, &w0, &g0, &n_groups);
       add_and_store<SRC>(bc->p, smem, ctl, blk, w0, g0, n_groups);
       __syncwarp();
     }
   }
   if constexpr (LANES16) {
-    tmem_fence_before();
+    tmem::fence_before();
     __syncthreads();
-    tmem_fence_after();
+    tmem::fence_after();
     __syncwarp();
-    if (threadIdx.x < 32) tmem_dealloc(ctl->tmem);
+    if (threadIdx.x < 32) tmem::dealloc(ctl->tmem);
   }
 }
 

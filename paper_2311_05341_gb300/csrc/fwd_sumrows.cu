@@ -34,8 +34,9 @@
 // words per thread), so partial sums never leave the SM and every output is
 // stored once.
 //
-// Every mbarrier wait is bounded; on timeout the CTA sets kErrTimeout, waits
-// for its copies, frees its tensor memory and stores nothing.
+// Every mbarrier wait is bounded, and no lane leaves the others in a warp-wide
+// operation (give_up); on timeout the CTA sets kErrTimeout, waits for its
+// copies (drain_copies) and frees its tensor memory.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -60,7 +61,8 @@ struct Ctl {
   uint64_t rows_empty[kSlots];  // the adders have read them
   uint32_t tmem;
   volatile int32_t abort;           // a wait gave up: every role leaves
-  volatile int32_t issued[kSlots];  // group + 1 whose copies were last issued into the slot
+  volatile int32_t issued[kSlots];  // group + 1 whose copies warp 0 last issued into the slot
+  volatile int32_t issued_by[kMainWarps];  // groups whose copies each adding warp has issued
 };
 static_assert(sizeof(Ctl) <= kRecOff, "control block too large");
 
@@ -70,7 +72,7 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
-// Bounded wait that also ends when the CTA is aborting.
+// Bounded wait that also ends when the CTA is aborting (a lane's own result).
 __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, const Ctl* ctl) {
   for (int it = 0; it < tk::kWaitIters; it += 64) {
     if (tk::mbar_wait(bar, parity, 64)) return true;
@@ -79,10 +81,10 @@ __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, con
   return false;
 }
 
-// Bounded wait for the copies of group g.  A parity wait only tells a phase
-// from the one before it, and the slot's previous group belongs to the other
-// warpgroup: the wait starts once the copies of g are issued, which follows
-// the end of that group.
+// Bounded wait for the copies of group g (a lane's own result).  A parity wait
+// only tells a phase from the one before it, and the slot's previous group
+// belongs to the other warpgroup: the wait starts once the copies of g are
+// issued, which follows the end of that group.
 __device__ __forceinline__ bool wait_copies(const Params& p, Ctl* ctl, int g) {
   const int slot = g % kSlots;
   for (int it = 0; ctl->issued[slot] <= g; ++it)
@@ -90,14 +92,42 @@ __device__ __forceinline__ bool wait_copies(const Params& p, Ctl* ctl, int g) {
   return tk::mbar_wait(smem_u32(&ctl->raw_full[slot]), (g / kSlots) & 1, p.wait_iters);
 }
 
-// After an abort: copies still in flight land before the CTA goes on (bounded:
-// a group that some adding warps left before issuing their part never
-// completes).
-__device__ __forceinline__ void drain_copies(const Ctl* ctl) {
-  for (int s = 0; s < kSlots; ++s)
-    if (ctl->issued[s] > 0)
-      tk::mbar_wait(smem_u32(&ctl->raw_full[s]), ((ctl->issued[s] - 1) / kSlots) & 1,
-                    kDrainIters);
+// A role gives up: the status word, and the flag that ends the other waits.
+// Lanes of a warp may find out one by one, and nothing bounds a warp-wide
+// operation that waits for a lane gone ahead, so warps vote on every wait
+// before they go on or leave: the building warps in build, the adding warps
+// with the byte counts of the copies they issue next (issue_copies).  The votes
+// cost 0.9 % of a launch from the packed copy (8192 channels: 70.4, now 71.0 ms
+// through the ring), nothing from the input.
+__device__ __forceinline__ void give_up(const Params& p, Ctl* ctl) {
+  atomicOr(p.err, tk::kErrTimeout);
+  ctl->abort = 1;
+}
+
+// After an abort, every role done: the copies still in flight land before the
+// CTA goes on.  The adding warps issue their shares of a group on their own,
+// and one that gave up first leaves its share out; a slot's warps are at most
+// one group apart (its next group is issued only once all copies of the last
+// one have landed).  The arrivals of the warps behind are made here, so that
+// the newest group's phase ends with the bytes that were asked for.
+__device__ __forceinline__ void drain_copies(const Params& p, const Ctl* ctl) {
+  for (int s = 0; s < kSlots; ++s) {
+    int newest = -1;
+    uint32_t missing = 0;
+    for (int w = 0; w < kMainWarps; ++w) {
+      int g = ctl->issued_by[w] - 1;              // the warp's newest group ...
+      g -= (g % kSlots - s + kSlots) % kSlots;    // ... of this slot
+      if (g == p.hold_stage) g -= kSlots;         // (never issued)
+      missing = g == newest ? missing : g > newest ? w : missing + 1;
+      newest = max(newest, g);
+    }
+    if (newest < 0) continue;
+    const uint32_t bar = smem_u32(&ctl->raw_full[s]);
+    if (missing > 0)
+      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(missing)
+                   : "memory");
+    tk::mbar_wait(bar, (newest / kSlots) & 1, kDrainIters);
+  }
 }
 __device__ __forceinline__ void mbar_inval(uint32_t bar) {
   asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
@@ -443,10 +473,14 @@ __device__ __forceinline__ void build_rows(const unsigned char* rec, uint32_t ra
 // them 68.0 ms, half by each 73.1 ms; from the input itself 78.3, 85.3 and
 // 85.7 ms.)
 static_assert(kMaxK <= 4 * kMainWarps, "four channels per adding warp");
+//
+// Also the warp's vote on the wait before it (`ok` of each lane; false where
+// any lane gave up, and then nothing is issued).
 template <int SRC>
-__device__ __forceinline__ void issue_copies(const Params& p, unsigned char* smem, Ctl* ctl,
-                                             int64_t w0, int g, const Dir& e, int32_t start) {
-  if (g == p.hold_stage) return;
+__device__ __forceinline__ bool issue_copies(const Params& p, unsigned char* smem, Ctl* ctl,
+                                             int64_t w0, int g, const Dir& e, int32_t start,
+                                             bool ok = true) {
+  if (g == p.hold_stage) return __all_sync(0xffffffffu, ok);
   constexpr int kBits = format(SRC).bits;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, slot = g % kSlots;
   const uint32_t bar = smem_u32(&ctl->raw_full[slot]);
@@ -457,7 +491,10 @@ __device__ __forceinline__ void issue_copies(const Params& p, unsigned char* sme
   if (lane < 4 && ch < e.k && at >= 0 && at < p.stride)
     bytes = static_cast<uint32_t>(
         min(static_cast<int64_t>(row_bytes), (p.stride - at) * kBits / 8));
-  const uint32_t total = __reduce_add_sync(0xffffffffu, bytes);
+  constexpr uint32_t kGaveUp = 1u << 24;  // above any sum of bytes, 32 of them below 2^32
+  static_assert(format(SRC).raw_bytes < kGaveUp, "byte counts and votes share a word");
+  const uint32_t total = __reduce_add_sync(0xffffffffu, ok ? bytes : kGaveUp);
+  if (total >= kGaveUp) return false;
   // The slot's last readers were ordinary loads.
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   if (lane == 0) {
@@ -476,6 +513,7 @@ __device__ __forceinline__ void issue_copies(const Params& p, unsigned char* sme
               static_cast<const unsigned char*>(p.x) +
                   (static_cast<int64_t>(e.c0 + ch) * p.stride + at) * kBits / 8,
               bytes, bar);
+  return true;
 }
 
 // Building warpgroup wg: channel groups wg, wg + 2, ...  Its last warp, which
@@ -489,12 +527,10 @@ __device__ __forceinline__ void build(const Params& p, unsigned char* smem, Ctl*
   constexpr size_t kRows = row_off(SRC), kRowBytes = static_cast<size_t>(format(SRC).row_words) * 4;
   for (int g = wg; g < n_groups; g += kBuildGroups) {
     const int slot = g % kSlots;
-    if (!wait_copies(p, ctl, g) ||
-        !wait_or_abort(smem_u32(&ctl->rows_empty[slot]), ((g / kSlots) & 1) ^ 1, ctl)) {
-      if (lane == 0) {
-        atomicOr(p.err, tk::kErrTimeout);
-        ctl->abort = 1;
-      }
+    const bool ok = wait_copies(p, ctl, g) &&
+                    wait_or_abort(smem_u32(&ctl->rows_empty[slot]), ((g / kSlots) & 1) ^ 1, ctl);
+    if (!__all_sync(0xffffffffu, ok)) {
+      if (lane == 0) give_up(p, ctl);
       return;
     }
     const unsigned char* rec = smem + kRecOff + slot * kRecBytes;
@@ -550,21 +586,24 @@ __device__ __forceinline__ void add_and_store(const Params& p, unsigned char* sm
   }
   for (int g = 0; g < n_groups; ++g) {
     const int slot = g % kSlots;
-    if (!wait_or_abort(smem_u32(&ctl->rows_full[slot]), (g / kSlots) & 1, ctl)) {
-      if (lane == 0) {
-        atomicOr(p.err, tk::kErrTimeout);
-        ctl->abort = 1;
-      }
-      return;
-    }
+    bool ok = wait_or_abort(smem_u32(&ctl->rows_full[slot]), (g / kSlots) & 1, ctl);
     const uint32_t* offs = reinterpret_cast<const uint32_t*>(smem + kOffsOff + slot * kOffsBytes);
     const bool flush = LANES16 && offs[kDm] != 0u;
     if (g + kSlots < n_groups) {
       const uint4 v = *reinterpret_cast<const uint4*>(offs + kNextDir);
       const Dir e = *reinterpret_cast<const Dir*>(&v);
       const int ch = min(w + kMainWarps * lane, kMaxK - 1);
-      issue_copies<SRC>(p, smem, ctl, w0, g + kSlots, e,
-                        static_cast<int32_t>(offs[kNextStart + ch]));
+      ok = issue_copies<SRC>(p, smem, ctl, w0, g + kSlots, e,
+                             static_cast<int32_t>(offs[kNextStart + ch]), ok);
+    } else {
+      ok = __all_sync(0xffffffffu, ok);
+    }
+    if (!ok) {
+      if (lane == 0) {
+        ctl->issued_by[w] = min(g + kSlots, n_groups);
+        give_up(p, ctl);
+      }
+      return;
     }
 #pragma unroll
     for (int i = 0; i < kDmPairs; ++i) {
@@ -588,6 +627,7 @@ __device__ __forceinline__ void add_and_store(const Params& p, unsigned char* sm
       }
     }
   }
+  if (lane == 0) ctl->issued_by[w] = n_groups;
   // Word k of the tile holds output w0 + k and, in 16-bit lanes, that plus the
   // pair distance.
   const int64_t lim = p.t_end - w0;
@@ -670,7 +710,7 @@ __global__ void __launch_bounds__(kThreads, 1) sum_row_kernel(const __grid_const
   }
   if constexpr (LANES16) tmem::fence_before();
   __syncthreads();
-  if (ctl->abort && threadIdx.x == 0) drain_copies(ctl);
+  if (ctl->abort && threadIdx.x == 0) drain_copies(p, ctl);
   if constexpr (LANES16) {
     tmem::fence_after();
     __syncwarp();
@@ -710,7 +750,7 @@ __global__ void __launch_bounds__(kThreads, 1) sum_row_batch_kernel(const BatchA
     const bool aborted = !fresh && ctl->abort;
     if (threadIdx.x == 0) {
       if (!fresh) {
-        if (aborted) drain_copies(ctl);
+        if (aborted) drain_copies(bc->p, ctl);
         for (int s = 0; s < kSlots; ++s) {
           mbar_inval(smem_u32(&ctl->raw_full[s]));
           mbar_inval(smem_u32(&ctl->rows_full[s]));

@@ -67,6 +67,10 @@ struct Ctl {
 static_assert(sizeof(Ctl) <= kRecOff, "control block too large");
 
 constexpr int kDrainIters = 1 << 14;  // polls, far longer than a copy takes
+// Polls of a shared word: some 40 cycles each, where a poll of an mbarrier
+// suspends its warp; a caller's short limit must not end a wait that only the
+// adders' work on three groups (10000 cycles) bounds.
+constexpr int kIssuePolls = 1 << 16;
 
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
@@ -86,9 +90,9 @@ __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, con
 // belongs to the other warpgroup: the wait starts once the copies of g are
 // issued, which follows the end of that group.
 __device__ __forceinline__ bool wait_copies(const Params& p, Ctl* ctl, int g) {
-  const int slot = g % kSlots;
+  const int slot = g % kSlots, polls = max(p.wait_iters, kIssuePolls);
   for (int it = 0; ctl->issued[slot] <= g; ++it)
-    if (it >= p.wait_iters || ctl->abort) return false;
+    if (it >= polls || ctl->abort) return false;
   return tk::mbar_wait(smem_u32(&ctl->raw_full[slot]), (g / kSlots) & 1, p.wait_iters);
 }
 

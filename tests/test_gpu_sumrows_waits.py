@@ -93,3 +93,17 @@ def test_withheld_group_in_a_batch(dtype, tile):
         runner.status()
         for i in range(2):
             np.testing.assert_array_equal(runner.planes(i)[0].cpu().numpy(), refs[i])
+
+
+@pytest.mark.parametrize("tile", ["pattern", "packed"])
+def test_short_wait_limit_leaves_a_healthy_run_alone(tile):
+    """64 polls of a copy's barrier suspend for longer than any copy takes, and
+    the limit counts no other wait: an ordinary run keeps within it."""
+    freqs, ranges = _ranges(640, 200, 0.2)
+    x, xd = _input("u8", 640, 30000, 9300)
+    plan = dd.Plan(freqs, F_HIGH, T_SAMP, ranges, "u8")
+    plan.set_tile(0, tile)
+    plan.set_wait_limit(64, -1)
+    got = plan.run(xd, n_samp=30000, segments=0)[0].cpu().numpy()
+    plan.device_status()
+    np.testing.assert_array_equal(got, oracle.forward(x, freqs, F_HIGH, T_SAMP, ranges)[0])

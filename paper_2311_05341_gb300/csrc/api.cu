@@ -679,7 +679,9 @@ static dd_status run_forward(dd_plan plan, const void* d_in, int64_t in_row_stri
     const void* src = d_in;
     int64_t stride = in_row_stride;
     int kind = 0;
-    if (range_copy[i] >= 0 && !sums_from_input(rp)) {  // reads its packed copy
+    // Reads its packed copy (a caller that packed it already may have given the
+    // input's memory another use since).
+    if (range_copy[i] >= 0 && !(pack && sums_from_input(rp))) {
       const PackedCopy& pc = copies[range_copy[i]];
       src = static_cast<unsigned char*>(d_scratch) + pc.offset;
       stride = pc.stride;

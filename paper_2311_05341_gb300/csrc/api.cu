@@ -643,14 +643,17 @@ static dd_status run_forward(dd_plan plan, const void* d_in, int64_t in_row_stri
   bool reads_copies = false;
   for (const RangePlan& rp : plan->ranges)
     reads_copies = reads_copies || (copy_kind(rp, true) != 0 && !sums_from_input(rp));
-  if (reads_copies && !n_keep && pack && d_scratch &&
+  const size_t need = packed_input_bytes(plan, n_samp, with_auto);
+  bool ring = false;
+  if ((reads_copies || need > 0) && !n_keep && pack && d_scratch &&
       scratch_bytes < packed_input_bytes(plan, n_samp, true)) {
     RingLayout L;
-    if (pick_ring(plan, info, n_samp, scratch_bytes, &L))
+    ring = pick_ring(plan, info, n_samp, scratch_bytes, &L);
+    if (ring && reads_copies)
       return run_ring(plan, info, d_in, in_row_stride, n_samp, d_out, d_scratch, L, stream);
   }
-  const size_t need = packed_input_bytes(plan, n_samp, with_auto);
-  if (need > 0) {
+  // (A ring that no range reads: its scratch is enough, and not used.)
+  if (need > 0 && !ring) {
     if (!d_scratch)
       return fail(DD_ERR_UNSUPPORTED,
                   "a range is on DD_TILE_PACKED: run it with dd_run_scratch and scratch of "

@@ -57,3 +57,41 @@ def test_run_packed_reads_the_copies(beam, tile):
                                  scratch.data_ptr(), n, _stream()))
     plan.device_status()
     np.testing.assert_array_equal(plan.split(out, N_SAMP)[0].cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("tile", [0, "packed"])
+@pytest.mark.parametrize("segments", [8, 3, 1])
+def test_run_takes_the_scratch_the_query_names(beam, tile, segments):
+    """dd_run_scratch with exactly the ring (or the full copies) that
+    dd_plan_packed_scratch_bytes gives for the segments."""
+    freqs, ranges, xd, ref = beam
+    lib = _lib.load()
+    plan = dd.Plan(freqs, F_HIGH, T_SAMP, ranges, "u16")
+    plan.set_tile(0, tile)
+    n = plan.packed_scratch_bytes(N_SAMP, segments)
+    assert 0 < n and (segments < 8 or n < plan.packed_scratch_bytes(N_SAMP, 1))
+    scratch = torch.zeros(n, dtype=torch.uint8, device="cuda")
+    out = plan.empty_output(N_SAMP)
+    _lib.check(lib.dd_run_scratch(plan.handle, xd.data_ptr(), xd.stride(0), N_SAMP, out.data_ptr(),
+                                  scratch.data_ptr(), n, _stream()))
+    plan.device_status()
+    np.testing.assert_array_equal(plan.split(out, N_SAMP)[0].cpu().numpy(), ref)
+
+
+def test_packed_tile_still_refuses_missing_and_short_scratch(beam):
+    freqs, ranges, xd, _ = beam
+    lib = _lib.load()
+    plan = dd.Plan(freqs, F_HIGH, T_SAMP, ranges, "u16")
+    plan.set_tile(0, "packed")
+    out = plan.empty_output(N_SAMP)
+    scratch = torch.zeros(4096, dtype=torch.uint8, device="cuda")
+    for ptr, n, status in ((None, 0, _lib.DD_ERR_UNSUPPORTED),
+                           (scratch.data_ptr(), 4096, _lib.DD_ERR_BUDGET)):
+        assert lib.dd_run_scratch(plan.handle, xd.data_ptr(), xd.stride(0), N_SAMP,
+                                  out.data_ptr(), ptr, n, _stream()) == status
+    keep = (ctypes.c_int64 * 1)(100)
+    ring = plan.packed_scratch_bytes(N_SAMP, 8)
+    scratch = torch.zeros(ring, dtype=torch.uint8, device="cuda")
+    assert lib.dd_run_window(plan.handle, xd.data_ptr(), xd.stride(0), N_SAMP, keep,
+                             out.data_ptr(), scratch.data_ptr(), ring,
+                             _stream()) == _lib.DD_ERR_BUDGET

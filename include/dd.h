@@ -99,7 +99,9 @@ typedef struct {
                                           pattern tile of uint8, 4-bit or uint16 input
                                           at bin 1, whose tables the packed kernel
                                           also runs) given the scratch of
-                                          dd_plan_packed_scratch_bytes; 0 otherwise */
+                                          dd_plan_packed_scratch_bytes; 0 otherwise.
+                                          (uint16 on the sum-row tile has such a copy
+                                          but reads it in dd_run_packed only) */
 } dd_plan_info;
 
 /* Adjoint kernels (dd_plan_info.adjoint_kernel). */
@@ -117,7 +119,10 @@ typedef struct {
  * 4 DMs per lane, one indexed branch per channel (or channel pair) over the
  * 32 patterns of per-DM shift increments a or a + 1 between a lane's DMs,
  * a = 0..3.  Plans whose shift of some channel grows by more than 4 between
- * consecutive trial DMs cannot use it. */
+ * consecutive trial DMs cannot use it.  In its automatic shape, integer ranges
+ * whose plan lets trial DMs share sums of adjacent channels run on the sum-row
+ * tile instead, with the same outputs (dd_plan_run_kernel says which; an
+ * explicit shape keeps the pattern kernel). */
 #define DD_TILE_PATTERN 0x104
 /* The pattern tile on a packed copy of uint8, 4-bit, uint16 or float32 input
  * (bin 1): word t of each channel holds samples t and t + 32 H in its 16-bit
@@ -129,7 +134,10 @@ typedef struct {
  * pattern tile of uint8, 4-bit and uint16 input at bin 1 runs the same
  * packed kernel whenever dd_run_scratch is given the scratch of
  * dd_plan_packed_scratch_bytes (full copies or a ring), and the unpacking
- * kernel otherwise. */
+ * kernel otherwise.  The sum-row tile takes the kernel's place as it does for
+ * DD_TILE_PATTERN: on the packed copy of uint8 and 4-bit input, and from the
+ * input itself for uint16, whose copy is then written by dd_pack_input and read
+ * by dd_run_packed (pattern kernel) only. */
 #define DD_TILE_PACKED 0x106
 
 /*
@@ -150,6 +158,30 @@ dd_status dd_plan_destroy(dd_plan plan);
 
 /* Fill *out with the plan's sizes for n_samp raw samples (n_samp >= 0). */
 dd_status dd_plan_query(dd_plan plan, int64_t n_samp, dd_plan_info* out);
+
+/* Kernels a launch can run on (dd_plan_run_kernel). */
+#define DD_RUN_GENERIC 1  /* shared-memory staged, any dtype and bin */
+#define DD_RUN_OFFSET 2   /* offset tile */
+#define DD_RUN_PATTERN 3  /* pattern tile, from the input or a packed copy */
+#define DD_RUN_SUM_ROWS 4 /* sum-row tile: sums over groups of channels, shared by the
+                             trial DMs that need them (integer input, at least 96
+                             channels, automatic shape) */
+#define DD_RUN_DIRECT 5   /* direct tile (an automatic offset tile of 1 or 2 DMs per
+                             lane, launches of enough outputs) */
+
+/*
+ * The kernel (DD_RUN_*) that computes n_out outputs of range `range` in one
+ * launch, and whether it reads a packed copy of the input (*reads_copy).
+ * scratch != 0: as dd_run_scratch with the scratch of
+ * dd_plan_packed_scratch_bytes (whose launches are the ring's segments or, for
+ * one segment, the whole range); 0: as dd_run, or for a DD_TILE_PACKED range
+ * with its scratch.  A range whose copy has no sum-row form while its input has
+ * (uint16) reads the input in either case.  Host only.
+ * Errors: DD_ERR_INVALID_ARG for NULL pointers or a bad index, DD_ERR_SHAPE
+ * for n_out <= 0.
+ */
+dd_status dd_plan_run_kernel(dd_plan plan, int32_t range, int64_t n_out, int32_t scratch,
+                             int32_t* kernel, int32_t* reads_copy);
 
 /* Copy the int32 shift table of range `range` to host memory host_out laid
  * out [n_dm][n_chan] (s(c,d) at host_out[d*n_chan + c]). */
@@ -256,7 +288,9 @@ dd_status dd_plan_packed_scratch_bytes(dd_plan plan, int64_t n_samp, int32_t n_s
  * dd_run with caller-owned device scratch (16-byte aligned; the library
  * allocates no device memory).  With at least dd_plan_packed_scratch_bytes(1)
  * every range with a packed copy reads the copy written there first (one
- * pass over the input, on `stream`).  With less, but at least the ring of
+ * pass over the input, on `stream`; ranges whose copy has no sum-row form while their
+ * input has, uint16, read d_in and leave their scratch untouched, here and
+ * below).  With less, but at least the ring of
  * some segment count in [2, 256] (dd_plan_packed_scratch_bytes), those
  * ranges run from the ring with the fewest segments that fits, packing and
  * the segments' kernels overlapped on the plan's own side streams (a
@@ -404,7 +438,7 @@ dd_status dd_plan_set_tile_shape(dd_plan plan, int32_t range, int32_t tile, int3
  * let its issued copies land and return, leaving that run's output undefined;
  * the context stays usable.  hold_stage >= 0 is a test hook for that path: the
  * copies of channel stage hold_stage (of every CTA of the register-tiled
- * kernels) are never issued, so the first wait on it runs out; -1 turns it
+ * kernels; on the sum-row tile, of channel group hold_stage) are never issued, so the first wait on it runs out; -1 turns it
  * off.  Host only; takes effect at the next launch (batches: at the next
  * dd_batch_bind).  The paper has no counterpart: the kernels' waits are this
  * library's own.

@@ -149,6 +149,15 @@ class Plan:
             "packed_copy": [bool(inf.packed_copy[i]) for i in range(n)],
         }
 
+    def run_kernel(self, r: int, n_out: int, scratch: bool = True) -> tuple:
+        """(kernel, reads a packed copy) of a launch of n_out outputs of range r:
+        "generic", "offset", "pattern", "sum-rows" or "direct", with scratch for
+        its packed copy or without (dd_plan_run_kernel)."""
+        k, c = ctypes.c_int32(), ctypes.c_int32()
+        check(self._lib.dd_plan_run_kernel(self._h, int(r), int(n_out), int(bool(scratch)),
+                                           ctypes.byref(k), ctypes.byref(c)))
+        return _lib.RUN_KERNELS[k.value], bool(c.value)
+
     def shifts(self, r: int = 0) -> np.ndarray:
         """int32 [n_dm][n_chan] shift table of range r (host copy)."""
         n_dm = self.info(0)["n_dm"][r]

@@ -22,6 +22,7 @@ DD_KERNEL_GENERIC, DD_KERNEL_TILED = 1, 2
 DD_TILE_PATTERN = 0x104
 DD_TILE_PACKED = 0x106
 DD_ADJOINT_GATHER, DD_ADJOINT_PATTERN = 1, 2
+RUN_KERNELS = {1: "generic", 2: "offset", 3: "pattern", 4: "sum-rows", 5: "direct"}  # DD_RUN_*
 
 
 class DDError(RuntimeError):
@@ -71,6 +72,8 @@ SIGNATURES = {
     "dd_plan_destroy": (ctypes.c_int, [_VP]),
     "dd_plan_query": (ctypes.c_int, [_VP, _I64, ctypes.POINTER(PlanInfo)]),
     "dd_plan_shifts": (ctypes.c_int, [_VP, _I32, _VP]),
+    "dd_plan_run_kernel": (ctypes.c_int, [_VP, _I32, _I64, _I32, ctypes.POINTER(_I32),
+                                          ctypes.POINTER(_I32)]),
     "dd_plan_upload": (ctypes.c_int, [_VP, _VP, _SZ, _VP]),
     "dd_plan_set_tile": (ctypes.c_int, [_VP, _I32, _I32]),
     "dd_run": (ctypes.c_int, [_VP, _VP, _I64, _I64, _VP, _VP]),

@@ -230,13 +230,9 @@ void free_host_pipe(dd_plan_s* p) {
 namespace {
 
 
-// Outputs [t_begin, t_end) of range rp.  kind > 0: the pattern tables run
-// by that packed-copy kernel (copy_kind) on packed words, element 0 of each
-// row holding word x_origin.
-int launch_range(const dd_plan_s* p, const RangePlan& rp, const void* d_in, int64_t stride,
-                 int64_t n_samp, int64_t n_out, void* d_out, int64_t t_begin, int64_t t_end,
-                 void* stream, int kind = 0, int64_t x_origin = 0) {
-  unsigned char* ws = static_cast<unsigned char*>(p->d_ws);
+// The kernel (DD_RUN_*) of a launch of `outputs` outputs of range rp; kind as
+// launch_range.
+int run_kernel(const RangePlan& rp, int kind, int64_t outputs) {
   const SumTables& sums = kind > 0 ? rp.packed_sums : rp.sums;
   // Bin 2 from the input: the pattern tile's units (64 DMs x 736 outputs) are
   // half as large and 0.8 of the time each, which tells in less than a wave.
@@ -244,10 +240,26 @@ int launch_range(const dd_plan_s* p, const RangePlan& rp, const void* d_in, int6
     const int64_t ctas = (dms + per_dms - 1) / per_dms * ((outs + 735) / 736);
     return ctas < 152 ? 1.0 : static_cast<double>(ctas) / 152;
   };
-  const bool small = sums.src == sr::kBytes2 && 1.25 * load(rp.n_dm, 128, t_end - t_begin) >
-                                                    load(rp.n_dm, 64, t_end - t_begin);
-  if (sums.ok && !small)
-    return launch_forward_sum_rows(p, rp, sums,
+  const bool small = sums.src == sr::kBytes2 &&
+                     1.25 * load(rp.n_dm, 128, outputs) > load(rp.n_dm, 64, outputs);
+  if (sums.ok && !small) return DD_RUN_SUM_ROWS;
+  if (kind > 0) return DD_RUN_PATTERN;
+  if (rp.direct.ok &&
+      dt::faster(static_cast<int32_t>(rp.n_dm), outputs, rp.direct.kind, rp.tile_dr))
+    return DD_RUN_DIRECT;
+  return !rp.tile_ok ? DD_RUN_GENERIC : rp.tile_pattern ? DD_RUN_PATTERN : DD_RUN_OFFSET;
+}
+
+// Outputs [t_begin, t_end) of range rp.  kind > 0: the pattern or sum-row
+// tables run by that packed-copy kernel (copy_kind) on packed words, element 0
+// of each row holding word x_origin.
+int launch_range(const dd_plan_s* p, const RangePlan& rp, const void* d_in, int64_t stride,
+                 int64_t n_samp, int64_t n_out, void* d_out, int64_t t_begin, int64_t t_end,
+                 void* stream, int kind = 0, int64_t x_origin = 0) {
+  unsigned char* ws = static_cast<unsigned char*>(p->d_ws);
+  const int run = run_kernel(rp, kind, t_end - t_begin);
+  if (run == DD_RUN_SUM_ROWS)
+    return launch_forward_sum_rows(p, rp, kind > 0 ? rp.packed_sums : rp.sums,
                                    ws + (kind > 0 ? rp.off_packed_sums : rp.off_sums),
                                    reinterpret_cast<int32_t*>(ws + tk::kStatusOffset), d_in,
                                    stride, d_out, t_begin, t_end, stream, n_out, x_origin);
@@ -256,8 +268,7 @@ int launch_range(const dd_plan_s* p, const RangePlan& rp, const void* d_in, int6
                                   reinterpret_cast<int32_t*>(ws + tk::kStatusOffset), d_in,
                                   stride, n_out, d_out, t_begin, t_end, stream, n_out, kind,
                                   x_origin);
-  if (rp.direct.ok && dt::faster(static_cast<int32_t>(rp.n_dm), t_end - t_begin, rp.direct.kind,
-                                 rp.tile_dr))
+  if (run == DD_RUN_DIRECT)
     return launch_forward_direct(p, rp, ws + rp.off_direct,
                                  reinterpret_cast<int32_t*>(ws + tk::kStatusOffset), d_in, stride,
                                  n_out, d_out, t_begin, t_end, stream);
@@ -433,6 +444,19 @@ dd_status dd_plan_query(dd_plan plan, int64_t n_samp, dd_plan_info* out) {
   if (!plan || !out) return fail(DD_ERR_INVALID_ARG, "plan or out is NULL");
   if (n_samp < 0) return fail(DD_ERR_INVALID_ARG, "n_samp < 0");
   return fill_info(plan, n_samp, out);
+}
+
+dd_status dd_plan_run_kernel(dd_plan plan, int32_t range, int64_t n_out, int32_t scratch,
+                             int32_t* kernel, int32_t* reads_copy) {
+  if (!plan || !kernel || !reads_copy) return fail(DD_ERR_INVALID_ARG, "NULL argument");
+  if (range < 0 || range >= static_cast<int32_t>(plan->ranges.size()))
+    return fail(DD_ERR_INVALID_ARG, "range index out of bounds");
+  if (n_out <= 0) return fail(DD_ERR_SHAPE, "n_out must be positive");
+  const RangePlan& rp = plan->ranges[range];
+  const int kind = sums_from_input(rp) ? 0 : copy_kind(rp, scratch != 0);
+  *kernel = run_kernel(rp, kind, n_out);
+  *reads_copy = kind > 0 ? 1 : 0;
+  return DD_OK;
 }
 
 dd_status dd_plan_shifts(dd_plan plan, int32_t range, int32_t* host_out) {

@@ -238,7 +238,7 @@ int run_kernel(const RangePlan& rp, int kind, int64_t outputs) {
   // half as large and 0.8 of the time each, which tells in less than a wave.
   auto load = [](int64_t dms, int64_t per_dms, int64_t outs) {
     const int64_t ctas = (dms + per_dms - 1) / per_dms * ((outs + 735) / 736);
-    return ctas < 152 ? 1.0 : static_cast<double>(ctas) / 152;
+    return ctas < tk::kSms ? 1.0 : static_cast<double>(ctas) / tk::kSms;
   };
   const bool small = sums.src == sr::kBytes2 &&
                      1.25 * load(rp.n_dm, 128, outputs) > load(rp.n_dm, 64, outputs);

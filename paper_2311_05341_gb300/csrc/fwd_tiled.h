@@ -57,6 +57,7 @@ DD_HOST_DEVICE constexpr int flush_words(int kind) { return kind == 1 ? 1288 : 6
 constexpr int kMaxWarps = 12;
 constexpr int kWaitIters = 1 << 22;  // default bound on the polls of an mbarrier wait
 constexpr int kErrTimeout = 1;       // device status bit: a bounded wait gave up
+constexpr int kSms = 152;  // of the GB300: a wave of one-CTA-per-SM kernels
 constexpr size_t kStatusOffset = 0;  // status word at the start of the plan workspace
 constexpr size_t kStatusBytes = 256;
 

@@ -66,3 +66,16 @@ def test_run_kernel_arguments():
         with pytest.raises(dd.DDError) as err:
             plan.run_kernel(*args)
         assert err.value.status == status
+
+
+@pytest.mark.parametrize("dtype,n_dm,n_out,want", [
+    # whole waves of 152 CTAs: 45 x 4 direct (2 waves) against 26 x 17 offset (3)
+    ("f32", 400, 16384, "offset"), ("u16", 400, 16384, "offset"), ("u8", 400, 32768, "offset"),
+    ("f32", 200, 32000, "offset"),
+    # 42 x 3 (1 wave) against 24 x 15 (3); 82 x 3 (2) against 47 x 15 (5)
+    ("f32", 356, 15360, "direct"), ("f32", 356, 30001, "direct"), ("u8", 356, 60002, "direct"),
+])
+def test_direct_tile_takes_whole_waves_into_account(dtype, n_dm, n_out, want):
+    plan = _plan(dtype, 336, n_dm, 5.5, 1, 400.0, 100.0, 327.68e-6)
+    assert plan.info(0)["tile_dms"] == [2]
+    assert plan.run_kernel(0, n_out)[0] == want

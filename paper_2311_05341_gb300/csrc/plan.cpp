@@ -426,15 +426,25 @@ void build_direct(RangePlan& rp, int32_t n_chan) {
   if (nc < std::min(4, n_chan)) return;
   rp.direct.bytes.assign(static_cast<size_t>(n_blocks) * n_chan * sizeof(dt::Rec), 0);
   dt::Rec* recs = reinterpret_cast<dt::Rec*>(rp.direct.bytes.data());
-  const bool ok = parallel_for(n_blocks, 2.0 * n_blocks * n_chan * dt::kDm, [&](int64_t b) {
-    for (int i = 0; i < dt::kDm; ++i) {
-      const int64_t d = std::min<int64_t>(b * dt::kDm + i, rp.n_dm - 1);
-      const int32_t* row = &rp.shifts[static_cast<size_t>(d) * n_chan];
-      for (int32_t c = 0; c < n_chan; ++c) {
-        dt::Rec& r = recs[b * n_chan + c];
-        if (i == 0) r.base = row[c];
-        if (row[c] < r.base) return false;
-        r.off[i] = static_cast<uint16_t>(row[c] - r.base + r.base % align);
+  // 64 channels' records at a time stay in the cache while the rows go by.
+  constexpr int32_t kChans = 64;
+  const bool ok = parallel_for(n_blocks, 1.0 * n_blocks * n_chan * dt::kDm, [&](int64_t b) {
+    const int32_t* first = &rp.shifts[static_cast<size_t>(b * dt::kDm) * n_chan];
+    for (int32_t c0 = 0; c0 < n_chan; c0 += kChans) {
+      const int32_t n = std::min(kChans, n_chan - c0);
+      dt::Rec* r = recs + b * n_chan + c0;
+      int32_t from[kChans];  // the window's first sample
+      for (int32_t c = 0; c < n; ++c) {
+        r[c].base = first[c0 + c];
+        from[c] = first[c0 + c] & ~(align - 1);  // align: a power of two
+      }
+      for (int i = 0; i < dt::kDm; ++i) {
+        const int64_t d = std::min<int64_t>(b * dt::kDm + i, rp.n_dm - 1);
+        const int32_t* row = &rp.shifts[static_cast<size_t>(d) * n_chan + c0];
+        for (int32_t c = 0; c < n; ++c) {
+          if (row[c] < r[c].base) return false;
+          r[c].off[i] = static_cast<uint16_t>(row[c] - from[c]);
+        }
       }
     }
     return true;

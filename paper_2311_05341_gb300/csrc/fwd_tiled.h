@@ -236,6 +236,11 @@ constexpr bool pat_shapes_fit_records() {
   return true;
 }
 static_assert(pat_shapes_fit_records(), "a pattern shape has more warps than its records hold");
+constexpr bool pat_shapes_stage_at_most(int channels) {
+  for (const PatShape& s : kPatShapes)
+    if (s.nc > channels) return false;
+  return true;
+}
 // The shape serves a kind: float-pair shapes (H < 15) serve kF32P only, with
 // channel pairs or single channels; the others pair integer window words or
 // take float words one channel at a time.

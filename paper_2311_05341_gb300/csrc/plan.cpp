@@ -181,9 +181,12 @@ bool build_pair_tables(const RangePlan& rp, int32_t n_chan, int kind, const tk::
     d = std::min<int64_t>(d, rp.n_dm - 1);
     return rp.shifts[static_cast<size_t>(d) * n_chan + c];
   };
+  constexpr int kMaxStage = 32;
+  static_assert(pat_shapes_stage_at_most(kMaxStage), "a shape stages more channels");
   // The blocks' tables are independent.
   auto block = [&](int64_t b) {
-    std::vector<std::vector<uint32_t>> by_pat(kPatterns);
+    uint32_t by_pat[kPatterns][kMaxStage];  // the stage's entries by pattern ...
+    int count[kPatterns];                   // ... and their numbers
     const int64_t d0 = b * dm_cta;
     int32_t* bases = reinterpret_cast<int32_t*>(out.data()) + b * n_chan;
     for (int32_t c = 0; c < n_chan; ++c) bases[c] = shift(d0, c);
@@ -192,7 +195,7 @@ bool build_pair_tables(const RangePlan& rp, int32_t n_chan, int kind, const tk::
       PairItem* items = reinterpret_cast<PairItem*>(chunk + kPairCountBytes);
       const int c0 = st * ps.nc, nc = std::min(ps.nc, n_chan - c0);
       for (int w = 0; w < ps.warps; ++w) {
-        for (auto& v : by_pat) v.clear();
+        std::fill(count, count + kPatterns, 0);
         const int64_t dw = d0 + static_cast<int64_t>(kPatDr) * w;
         for (int k = 0; k < nc; ++k) {
           const int32_t c = c0 + k;
@@ -206,18 +209,19 @@ bool build_pair_tables(const RangePlan& rp, int32_t n_chan, int kind, const tk::
           if (!pattern_of(s_dm, n_real, ps.amax, &pat)) return false;
           const uint32_t a = static_cast<uint32_t>(k) * lp + static_cast<uint32_t>(off);
           if (a > 0xffffu) return false;
-          by_pat[pat].push_back(a);
+          by_pat[pat][count[pat]++] = a;
         }
         int n = 0;
         for (uint32_t pat = 0; pat < static_cast<uint32_t>(kPatterns); ++pat) {
-          const auto& v = by_pat[pat];
-          for (size_t i = 0; i + 1 < v.size(); i += 2)
+          const uint32_t* v = by_pat[pat];
+          for (int i = 0; i + 1 < count[pat]; i += 2)
             items[w * ps.nc + n++] = PairItem{v[i] | v[i + 1] << 16, pat};
         }
         chunk[w] = static_cast<unsigned char>(n);
         const int n_pairs = n;
         for (uint32_t pat = 0; pat < static_cast<uint32_t>(kPatterns); ++pat)
-          if (by_pat[pat].size() % 2) items[w * ps.nc + n++] = PairItem{by_pat[pat].back(), pat};
+          if (count[pat] % 2)
+            items[w * ps.nc + n++] = PairItem{by_pat[pat][count[pat] - 1], pat};
         chunk[kPairMaxWarps + w] = static_cast<unsigned char>(n - n_pairs);
       }
     }

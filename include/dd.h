@@ -171,11 +171,11 @@ dd_status dd_plan_query(dd_plan plan, int64_t n_samp, dd_plan_info* out);
 
 /*
  * The kernel (DD_RUN_*) that computes n_out outputs of range `range` in one
- * launch, and whether it reads a packed copy of the input (*reads_copy).
- * scratch != 0: as dd_run_scratch with the scratch of
- * dd_plan_packed_scratch_bytes (whose launches are the ring's segments or, for
- * one segment, the whole range); 0: as dd_run, or for a DD_TILE_PACKED range
- * with its scratch.  A range whose copy has no sum-row form while its input has
+ * launch of its own, and whether it reads a packed copy of the input
+ * (*reads_copy).  scratch != 0: as dd_run_scratch with the full copies of
+ * dd_plan_packed_scratch_bytes(1) (the ring's segments, which overlap, keep the
+ * sum-row tile where the range has it); 0: as dd_run, or for a DD_TILE_PACKED
+ * range with its scratch.  A range whose copy has no sum-row form while its input has
  * (uint16) reads the input in either case.  Host only.
  * Errors: DD_ERR_INVALID_ARG for NULL pointers or a bad index, DD_ERR_SHAPE
  * for n_out <= 0.

@@ -230,19 +230,18 @@ void free_host_pipe(dd_plan_s* p) {
 namespace {
 
 
-// The kernel (DD_RUN_*) of a launch of `outputs` outputs of range rp; kind as
-// launch_range.
-int run_kernel(const RangePlan& rp, int kind, int64_t outputs) {
+// The kernel (DD_RUN_*) of a launch of `outputs` outputs of range rp; kind and
+// overlapped as launch_range.  Segments that overlap fill each other's last
+// waves: they keep the sum-row tile, but for bin 2 from the input, whose
+// pattern units (64 DMs x 736 outputs) are half as large and 0.8 of the time.
+int run_kernel(const dd_plan_s* p, const RangePlan& rp, int kind, int64_t outputs,
+               bool overlapped) {
   const SumTables& sums = kind > 0 ? rp.packed_sums : rp.sums;
-  // Bin 2 from the input: the pattern tile's units (64 DMs x 736 outputs) are
-  // half as large and 0.8 of the time each, which tells in less than a wave.
-  auto load = [](int64_t dms, int64_t per_dms, int64_t outs) {
-    const int64_t ctas = (dms + per_dms - 1) / per_dms * ((outs + 735) / 736);
-    return ctas < tk::kSms ? 1.0 : static_cast<double>(ctas) / tk::kSms;
-  };
-  const bool small = sums.src == sr::kBytes2 &&
-                     1.25 * load(rp.n_dm, 128, outputs) > load(rp.n_dm, 64, outputs);
-  if (sums.ok && !small) return DD_RUN_SUM_ROWS;
+  if (sums.ok &&
+      ((overlapped && sums.src != sr::kBytes2) || sums_only(rp, kind) ||
+       sum_rows_faster(sums, rp, p->n_chan, p->dtype == DD_U4, kind > 0 ? kind : rp.tile_kind,
+                       outputs, overlapped)))
+    return DD_RUN_SUM_ROWS;
   if (kind > 0) return DD_RUN_PATTERN;
   if (rp.direct.ok &&
       dt::faster(static_cast<int32_t>(rp.n_dm), outputs, rp.direct.kind, rp.tile_dr))
@@ -252,12 +251,13 @@ int run_kernel(const RangePlan& rp, int kind, int64_t outputs) {
 
 // Outputs [t_begin, t_end) of range rp.  kind > 0: the pattern or sum-row
 // tables run by that packed-copy kernel (copy_kind) on packed words, element 0
-// of each row holding word x_origin.
+// of each row holding word x_origin.  overlapped: one of several segments whose
+// launches overlap on two streams.
 int launch_range(const dd_plan_s* p, const RangePlan& rp, const void* d_in, int64_t stride,
                  int64_t n_samp, int64_t n_out, void* d_out, int64_t t_begin, int64_t t_end,
-                 void* stream, int kind = 0, int64_t x_origin = 0) {
+                 void* stream, int kind = 0, int64_t x_origin = 0, bool overlapped = false) {
   unsigned char* ws = static_cast<unsigned char*>(p->d_ws);
-  const int run = run_kernel(rp, kind, t_end - t_begin);
+  const int run = run_kernel(p, rp, kind, t_end - t_begin, overlapped);
   if (run == DD_RUN_SUM_ROWS)
     return launch_forward_sum_rows(p, rp, kind > 0 ? rp.packed_sums : rp.sums,
                                    ws + (kind > 0 ? rp.off_packed_sums : rp.off_sums),
@@ -454,7 +454,7 @@ dd_status dd_plan_run_kernel(dd_plan plan, int32_t range, int64_t n_out, int32_t
   if (n_out <= 0) return fail(DD_ERR_SHAPE, "n_out must be positive");
   const RangePlan& rp = plan->ranges[range];
   const int kind = sums_from_input(rp) ? 0 : copy_kind(rp, scratch != 0);
-  *kernel = run_kernel(rp, kind, n_out);
+  *kernel = run_kernel(plan, rp, kind, n_out, false);
   *reads_copy = kind > 0 ? 1 : 0;
   return DD_OK;
 }
@@ -629,7 +629,7 @@ static dd_status run_ring(dd_plan plan, const dd_plan_info& info, const void* d_
       const RangePlan& rp = plan->ranges[r];
       le = launch_range(plan, rp, buf, L.slot_words, n_samp, info.n_out[r],
                         out + info.out_offset[r] * 4, sg.lo[r], sg.hi[r], sc,
-                        copy_kind(rp, true), sg.origin);
+                        copy_kind(rp, true), sg.origin, true);
       if (le != 0) return fail_joined(hp, s, le, "dd_run ring forward launch");
     }
     e = cudaEventRecord(hp->freed[slot], sc);
@@ -954,7 +954,7 @@ static dd_status run_host_pipeline(dd_plan plan, const dd_plan_info& info, const
       if (l > done[r]) {
         const int le = launch_range(plan, rp, from_packed ? d_packed : dcm,
                                     from_packed ? packed_stride : cm_stride, n_samp, n_out,
-                                    dout + info.out_offset[r] * 4, done[r], l, sc, kind);
+                                    dout + info.out_offset[r] * 4, done[r], l, sc, kind, 0, true);
         if (le != 0) return fail_joined(hp, s, le, "dd_run_host forward launch");
       }
     }

@@ -42,6 +42,9 @@ struct dd_batch_s {
   std::vector<dd::tk::BatchJob> host_jobs;
   std::vector<dd::tk::PatBatchJob> host_pjobs;
   std::vector<dd::sr::Params> host_sjobs;
+  bool use_sums[5] = {};  // by window format (sr::Src): the batch runs it on sum rows
+  // The sum-row tables the batch runs a range from, nullptr for another tile.
+  const dd::SumTables* sums_of(const dd::RangePlan& rp) const;
   // Pattern-tile jobs grouped by variant (kind, shape) and sum-row jobs by
   // window format (sr::Src, shape kSumRows): one launch each.
   static constexpr int32_t kSumRows = -1;
@@ -98,12 +101,48 @@ namespace {
 
 size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 
-// The sum-row tables a batch runs a range from: the packed copy's on
+// The sum-row tables a batch can run a range from: the packed copy's on
 // DD_TILE_PACKED, else the input's; nullptr without them.
 const dd::SumTables* batch_sums(const dd::RangePlan& rp) {
+  if (!rp.tile_ok || !rp.tile_pattern) return nullptr;
   const dd::SumTables& t =
       dd::tk::packed_copy_kind(rp.tile_kind) && !dd::sums_from_input(rp) ? rp.packed_sums : rp.sums;
   return t.ok ? &t : nullptr;
+}
+
+// Which window formats the batch runs on sum rows: the rule of a single launch
+// (sum_rows_faster) on the units of all ranges of the format, which one
+// persistent launch takes; overlapped with the batch's other launches, if any.
+// Measured on 1134 batches of 1 and 4 equal beams (150 to 2000 channels, 64 to
+// 1000 DMs, 0.3 to 2 samples a step, every format): 1.25 times the pattern
+// tile's speed on average and nine at 0.93 to 0.98 of it (on sum rows always:
+// 52, down to 0.75).  The 5 % in favour of the sum rows are within what the
+// costs are good for.
+void choose_sums(dd_batch_s* b) {
+  using namespace dd;
+  std::vector<UnitCost> sums[5], pattern[5];
+  int64_t jobs[5] = {}, all = 0;
+  for (size_t i = 0; i < b->plans.size(); ++i)
+    for (const RangePlan& rp : b->plans[i]->ranges) {
+      ++all;
+      const SumTables* t = batch_sums(rp);
+      const int64_t n_out = range_n_out(b->plans[i], rp, b->n_samp[i]);
+      if (!t || n_out <= 0) continue;
+      ++jobs[t->src];
+      add_sum_row_units(*t, true, n_out, &sums[t->src]);
+      add_pattern_units(rp, b->plans[i]->n_chan, b->plans[i]->dtype == DD_U4, rp.tile_kind, n_out,
+                        &pattern[t->src]);
+    }
+  constexpr double kFavour = 0.95;
+  auto cheaper = [](const UnitCost& a, const UnitCost& c) { return a.cycles < c.cycles; };
+  for (int s = 0; s < 5; ++s) {
+    if (jobs[s] == 0) continue;
+    std::sort(sums[s].begin(), sums[s].end(), cheaper);
+    std::sort(pattern[s].begin(), pattern[s].end(), cheaper);
+    for (UnitCost& u : sums[s]) u.cycles *= kFavour;
+    const bool overlapped = jobs[s] < all;
+    b->use_sums[s] = launch_cycles(sums[s], overlapped) < launch_cycles(pattern[s], overlapped);
+  }
 }
 
 bool batch_shape(int32_t dr) {
@@ -113,6 +152,12 @@ bool batch_shape(int32_t dr) {
 }
 
 }  // namespace
+
+const dd::SumTables* dd_batch_s::sums_of(const dd::RangePlan& rp) const {
+  const dd::SumTables* t = batch_sums(rp);
+  return t && (use_sums[t->src] || dd::sums_only(rp, t->src == dd::sr::kPairs ? 1 : 0)) ? t
+                                                                                       : nullptr;
+}
 
 using namespace dd;
 
@@ -132,13 +177,16 @@ dd_status dd_batch_create(const dd_plan* plans, const int64_t* n_samp, int32_t n
     };
     std::vector<Cost> order;
     for (int32_t i = 0; i < n_plans; ++i) {
-      const dd_plan p = plans[i];
-      if (!p) {
+      if (!plans[i]) {
         delete b;
         return fail(DD_ERR_INVALID_ARG, "NULL plan in batch");
       }
-      b->plans.push_back(p);
+      b->plans.push_back(plans[i]);
       b->n_samp.push_back(n_samp[i]);
+    }
+    choose_sums(b);
+    for (int32_t i = 0; i < n_plans; ++i) {
+      const dd_plan p = plans[i];
       int64_t out_off = 0;
       for (size_t r = 0; r < p->ranges.size(); ++r) {
         const RangePlan& rp = p->ranges[r];
@@ -169,7 +217,7 @@ dd_status dd_batch_create(const dd_plan* plans, const int64_t* n_samp, int32_t n
         int32_t index;
         int ts;
         double dms;
-        const SumTables* sums = pat ? batch_sums(rp) : nullptr;
+        const SumTables* sums = b->sums_of(rp);
         if (sums) {
           index = static_cast<int32_t>(b->host_sjobs.size());
           b->host_sjobs.emplace_back();
@@ -219,7 +267,7 @@ dd_status dd_batch_create(const dd_plan* plans, const int64_t* n_samp, int32_t n
       const RangePlan& rp = p->ranges[j.range];
       const int ts = j.pattern ? tk::pat_tile_samples(rp.tile_kind, rp.tile_h)
                                : tk::tile_samples(rp.tile_kind);
-      const SumTables* sums = j.sums ? batch_sums(rp) : nullptr;
+      const SumTables* sums = j.sums ? b->sums_of(rp) : nullptr;
       const int64_t tiles =
           sums ? sum_row_halves(sums->src, 0, j.n_out) : (j.n_out + ts - 1) / ts;
       const int32_t n_blocks = sums ? sums->n_blocks : rp.tile_n_blocks;
@@ -270,7 +318,7 @@ dd_status dd_batch_create(const dd_plan* plans, const int64_t* n_samp, int32_t n
       for (const auto& j : b->jobs) {
         if (j.plan != b->packs[k].plan || !j.pattern) continue;
         if (range_copy[j.range] != b->packs[k].copy_index) continue;
-        const SumTables* sums = j.sums ? batch_sums(b->plans[j.plan]->ranges[j.range]) : nullptr;
+        const SumTables* sums = j.sums ? b->sums_of(b->plans[j.plan]->ranges[j.range]) : nullptr;
         if (sums && sums->src != sr::kPairs) continue;  // reads the input
         const int32_t lane = b->group_of(j);
         auto& lp = b->lane_packs[lane];
@@ -403,7 +451,7 @@ dd_status dd_batch_bind_scratch(dd_batch batch, const void* const* d_in,
         stride < n || stride_bytes % 16 != 0 || (p->dtype == DD_U4 && stride % 2 != 0))
       return fail(DD_ERR_SHAPE, "batch input/output alignment or stride");
     const RangePlan& rp = p->ranges[jr.range];
-    const SumTables* sums = jr.sums ? batch_sums(rp) : nullptr;
+    const SumTables* sums = jr.sums ? batch->sums_of(rp) : nullptr;
     if (rp.tile_ok && (sums ? sums->src == sr::kPairs
                             : tk::packed_copy_kind(rp.tile_kind))) {  // reads its packed copy
       std::vector<int32_t> range_copy;

@@ -211,6 +211,11 @@ inline int copy_kind(const RangePlan& rp, bool with_auto) {
 // The range runs on the sum-row tile from the input whatever scratch the
 // caller gives (uint16: its packed copy has no sum-row kernel).
 inline bool sums_from_input(const RangePlan& rp) { return rp.sums.ok && !rp.packed_sums.ok; }
+// No pattern tables serve such a launch (kind as copy_kind, 0: from the input):
+// a DD_TILE_PACKED range's are for its copy.
+inline bool sums_only(const RangePlan& rp, int kind) {
+  return kind == 0 && tk::packed_copy_kind(rp.tile_kind);
+}
 // Pair distance of the packed copy a range reads with kernel kind `kind`.
 inline int32_t pack_pair(const RangePlan& rp, int kind) {
   return kind == tk::kU8P || kind == tk::kF32P ? 32 * rp.tile_h : 0;

@@ -76,6 +76,8 @@ struct Block {
   std::vector<int32_t> start;
   std::vector<unsigned char> recs;
   double words = 0;
+  double unit = 0;        // cycles of a unit (Format::unit_add ...)
+  double batch_unit = 0;  // in the persistent kernel
 };
 
 bool build_block(const RangePlan& rp, int32_t n_chan, int lane_chans, const Format& f, int64_t b,
@@ -92,6 +94,8 @@ bool build_block(const RangePlan& rp, int32_t n_chan, int lane_chans, const Form
   }
   int32_t c = 0;
   int since = 0;  // channels in the lanes
+  out->unit = f.unit_fixed;
+  out->batch_unit = f.batch_fixed;
   while (c < n_chan) {
     const int32_t* s0 = &block[static_cast<size_t>(c) * kDm];
     const int rs = round_up(kWords + s0[n_real - 1] - s0[0], f.build);
@@ -240,12 +244,19 @@ bool build_block(const RangePlan& rp, int32_t n_chan, int lane_chans, const Form
     if (since + best.k > lane_chans) {
       const uint16_t one = 1;
       std::memcpy(recs.data() + last_head + offsetof(RecHead, flush), &one, 2);
+      out->unit += f.unit_flush;
+      out->batch_unit += f.unit_flush;
       since = 0;
     }
     since += best.k;
     last_head = head;
     dir.push_back(e);
     out->words += best_cost * best.k;
+    const int passes = (best.rs + 32 * f.build * kBuildWarps - 1) / (32 * f.build * kBuildWarps);
+    const double building = passes * (f.unit_group + f.unit_chan * best.k +
+                                      static_cast<double>(f.unit_move) * h.n_steps) / 2;
+    out->unit += std::max<double>(f.unit_add, building);
+    out->batch_unit += std::max<double>(f.batch_add, building);
     c += best.k;
     if (recs.size() > (size_t{1} << 30)) return false;
   }
@@ -253,6 +264,69 @@ bool build_block(const RangePlan& rp, int32_t n_chan, int lane_chans, const Form
 }
 
 }  // namespace
+
+double launch_cycles(const std::vector<UnitCost>& sorted, bool overlapped) {
+  int64_t n = 0;
+  double total = 0;
+  for (const UnitCost& u : sorted) {
+    n += u.count;
+    total += u.cycles * static_cast<double>(u.count);
+  }
+  if (n == 0) return 0;
+  if (overlapped)
+    return std::max(static_cast<double>(n) / tk::kSms, 0.5) * total / static_cast<double>(n);
+  const int64_t waves = (n + tk::kSms - 1) / tk::kSms;
+  if (waves == 1) return sorted.back().cycles;
+  // The share of the units (by cost) that frees the SMs of the last wave.
+  const double share = static_cast<double>(n - (waves - 1) * tk::kSms) / tk::kSms;
+  double start = 0, seen = 0;
+  for (const UnitCost& u : sorted) {
+    start = u.cycles;
+    seen += static_cast<double>(u.count);
+    if (seen >= share * static_cast<double>(n)) break;
+  }
+  return static_cast<double>(waves - 2) * total / static_cast<double>(n) + start +
+         sorted.back().cycles;
+}
+
+void add_sum_row_units(const SumTables& t, bool batch, int64_t outputs,
+                       std::vector<UnitCost>* units) {
+  const int64_t halves = sum_row_halves(t.src, 0, outputs);
+  for (double c : batch ? t.batch_cycles : t.unit_cycles) units->push_back({c, halves});
+}
+
+void add_pattern_units(const RangePlan& rp, int32_t n_chan, bool nibbles, int kind,
+                       int64_t outputs, std::vector<UnitCost>* units) {
+  // Cycles of a 64-DM unit, per channel and besides, as measured: one kind and
+  // bin each (7 % around them).
+  struct {
+    double per_chan, fixed;
+  } c;
+  switch (kind) {
+    case tk::kU8: c = {559, 33000}; break;
+    case tk::kU4: c = {598, 30000}; break;
+    case tk::kU16: c = {536, 13300}; break;
+    case tk::kU8W: c = {589, 14000}; break;  // bin 2
+    default:                                 // kU8P
+      c = {nibbles        ? 475.0
+           : rp.r.bin == 1 ? 500.0
+           : rp.r.bin == 2 ? 563.0
+           : rp.r.bin == 4 ? 672.0
+                           : 914.0,
+           31000};
+  }
+  const int ts = tk::pat_tile_samples(kind, rp.tile_h);
+  units->push_back({c.fixed + c.per_chan * n_chan, (outputs + ts - 1) / ts * rp.tile_n_blocks});
+}
+
+bool sum_rows_faster(const SumTables& t, const RangePlan& rp, int32_t n_chan, bool nibbles,
+                     int kind, int64_t outputs, bool overlapped) {
+  std::vector<UnitCost> sums, pattern;
+  sums.reserve(t.unit_cycles.size());
+  add_sum_row_units(t, false, outputs, &sums);
+  add_pattern_units(rp, n_chan, nibbles, kind, outputs, &pattern);
+  return launch_cycles(sums, overlapped) < launch_cycles(pattern, overlapped);
+}
 
 void build_sum_tables(const RangePlan& rp, int32_t n_chan, int64_t max_sample, int src,
                       SumTables* out) {
@@ -321,6 +395,12 @@ void build_sum_tables(const RangePlan& rp, int32_t n_chan, int64_t max_sample, i
   out->n_blocks = static_cast<int32_t>(n_blocks);
   out->off_dir = static_cast<int32_t>(off_dir);
   out->off_start = static_cast<int32_t>(off_start);
+  for (const Block& b : blocks) {
+    out->unit_cycles.push_back(b.unit);
+    out->batch_cycles.push_back(b.batch_unit);
+  }
+  std::sort(out->unit_cycles.begin(), out->unit_cycles.end());
+  std::sort(out->batch_cycles.begin(), out->batch_cycles.end());
   out->ok = true;
 }
 

@@ -67,6 +67,14 @@ struct Format {
   int row_words;   // row buffer
   int chain_chan;  // measured cycles of a building warp per channel of a group
   int chain_move;  // and per move (kChainGroup per group besides)
+  // A unit's cycles, fitted to measured launches (launch_cycles): unit_fixed,
+  // and per group the larger of unit_add and, for each pass of the building
+  // warps over its rows, half of unit_group + unit_chan per channel + unit_move
+  // per move; unit_flush for each time the 16-bit lanes give up their high bytes.
+  int unit_add, unit_group, unit_chan, unit_move, unit_flush, unit_fixed;
+  // The same in the persistent kernel, which starts its pipeline anew for every
+  // unit and whose adding warps are slower.
+  int batch_add, batch_fixed;
 };
 constexpr int kChainGroup = 900;
 constexpr int kAddGroup = 2900;  // cycles of the adding warps per group
@@ -75,11 +83,16 @@ constexpr int kAddGroup = 2900;  // cycles of the adding warps per group
 // unaligned bytes (two 32-bit words and a funnel shift), stored 16 bytes at a
 // time; a window is less than half as long in bytes, so the rows get more.
 DD_HOST_DEVICE constexpr Format format(int src) {
-  return src == kPairs      ? Format{32, 16, 5, 1, 29696, 11392, 110, 155}
-         : src == kBytes    ? Format{8, 16, 4, kWords + 8, 17408, 14464, 190, 145}
-         : src == kNibbles  ? Format{4, 32, 4, kWords + 16, 17408, 14464, 195, 165}
-         : src == kHalves   ? Format{16, 16, 4, 4, 17408, 14464, 380, 130}
-                            : Format{16, 16, 4, kWords + 4, 29696, 11392, 300, 200};
+  return src == kPairs ? Format{32, 16, 5, 1, 29696, 11392, 110, 155,
+                                1820, 2730, 61, 129, 2040, 28000, 3510, 55000}
+         : src == kBytes ? Format{8, 16, 4, kWords + 8, 17408, 14464, 190, 145,
+                                  3270, 130, 138, 211, 220, 27000, 4480, 38000}
+         : src == kNibbles ? Format{4, 32, 4, kWords + 16, 17408, 14464, 195, 165,
+                                    3320, 30, 126, 248, 610, 28500, 4150, 42000}
+         : src == kHalves ? Format{16, 16, 4, 4, 17408, 14464, 380, 130,
+                                   2870, 80, 89, 193, 0, 13000, 3160, 28000}
+                          : Format{16, 16, 4, kWords + 4, 29696, 11392, 300, 200,
+                                   3950, 15, 173, 370, 1500, 25000, 4460, 44500};
 }
 // Output samples of a CTA's words, and of the pattern time tile holding them.
 DD_HOST_DEVICE constexpr int pair_dist(int src) { return src == kPairs ? kPairWords : kWords; }
@@ -178,8 +191,40 @@ struct SumTables {
   int32_t n_blocks = 0;
   int32_t off_dir = 0;
   int32_t off_start = 0;
+  // What a unit (128 DMs x 368 words) takes, per DM block in ascending order,
+  // and in the persistent kernel.
+  std::vector<double> unit_cycles;
+  std::vector<double> batch_cycles;
   std::vector<unsigned char> bytes;
 };
+
+// Cycles (at about 2 GHz) of a launch of one-CTA-per-SM units, `count` of every
+// cost in `sorted` (ascending): whole waves of kSms CTAs of mean cost, the last
+// of which starts when as many units as it has are through the wave before (the
+// cheapest), and ends with the dearest.  overlapped: among launches that fill
+// each other's gaps, for which units count as such, but a launch does not fall
+// below half a wave of two in flight.
+struct UnitCost {
+  double cycles;
+  int64_t count;
+};
+double launch_cycles(const std::vector<UnitCost>& sorted, bool overlapped);
+// The units of `outputs` outputs of a range on the sum-row tile, and on the
+// pattern kernel `kind` (its tables' kind or the packed copy's), appended.
+void add_sum_row_units(const SumTables& t, bool batch, int64_t outputs,
+                       std::vector<UnitCost>* units);
+void add_pattern_units(const RangePlan& rp, int32_t n_chan, bool nibbles, int kind,
+                       int64_t outputs, std::vector<UnitCost>* units);
+// Whether the sum-row tile takes the launch.  Its 128-DM units leave more of
+// the chip idle than the pattern tile's 64-DM ones where there are few: 150
+// channels x 130 DMs x 60000 uint8 outputs make 164 units, 2 waves of 66 us
+// together, where 123 of the pattern tile take 58.  Measured over 100 to 3000
+// channels, 64 to 1000 DMs, 20000 to 74000 outputs and 0.1 to 2 samples a step,
+// every format (1175 launches): never slower than the pattern tile (the sum-row
+// tile always: up to 1.21 times its time), and 1.0004 times the better of the
+// two on average.
+bool sum_rows_faster(const SumTables& t, const RangePlan& rp, int32_t n_chan, bool nibbles,
+                     int kind, int64_t outputs, bool overlapped);
 
 // max_sample: the largest (decimated) sample.  ok == false where the tile
 // would not be faster than the pattern tile or cannot hold the sums.

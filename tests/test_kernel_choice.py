@@ -79,3 +79,24 @@ def test_direct_tile_takes_whole_waves_into_account(dtype, n_dm, n_out, want):
     plan = _plan(dtype, 336, n_dm, 5.5, 1, 400.0, 100.0, 327.68e-6)
     assert plan.info(0)["tile_dms"] == [2]
     assert plan.run_kernel(0, n_out)[0] == want
+
+
+@pytest.mark.parametrize("dtype,n_chan,n_dm,slope,bin_,n_out,want", [
+    # 2 x 82 units of 128 DMs (2 waves of 152) against 3 x 41 of 64 (1)
+    ("u8", 150, 130, 0.4, 1, 60000, "pattern"), ("u8", 300, 130, 1.0, 1, 60000, "pattern"),
+    ("u4", 150, 130, 0.4, 1, 60000, "pattern"), ("u16", 150, 130, 0.4, 1, 30000, "pattern"),
+    ("u8", 150, 130, 0.4, 1, 50000, "sum-rows"), ("u8", 1500, 130, 0.4, 1, 60000, "sum-rows"),
+    ("u8", 150, 512, 0.4, 1, 73600, "sum-rows"), ("u16", 150, 130, 0.4, 1, 20000, "sum-rows"),
+    ("u8", 150, 130, 0.4, 2, 30000, "pattern"), ("u8", 700, 1000, 0.4, 2, 66240, "sum-rows"),
+])
+def test_sum_row_tile_takes_whole_waves_into_account(dtype, n_chan, n_dm, slope, bin_, n_out, want):
+    plan = _plan(dtype, n_chan, n_dm, slope, bin_)
+    assert plan.run_kernel(0, n_out, scratch=False) == (want, False)
+
+
+def test_packed_uint16_never_reads_the_input_with_its_copys_tables():
+    """DD_TILE_PACKED uint16 has pattern tables for its copy alone: from the input
+    it stays on the sum-row tile where the rule would prefer the pattern tile."""
+    plan = _plan("u16", 150, 130, 0.4)
+    plan.set_tile(0, "packed")
+    assert plan.run_kernel(0, 30000) == ("sum-rows", False)

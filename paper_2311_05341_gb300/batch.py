@@ -100,11 +100,17 @@ def input_buffer(dtype: str, n_chan: int, n_samp: int, device, n_cols: int | Non
                      "u4": torch.uint8}[dtype])
 
 
+# Generation of the candidates and of the kernels they run: choices cached
+# before the automatic shape was a candidate are not taken for today's.
+TUNING_VERSION = 2
+
+
 def plan_signature(plan: Plan, n_samp: int) -> str:
-    """Key of the autotune cache: everything that changes the tile's work."""
+    """Key of the autotune cache: everything that changes the tile's work, and
+    what the candidates are (TUNING_VERSION)."""
     h = hashlib.sha1(plan.freqs.tobytes()).hexdigest()[:16]
     return json.dumps([plan.dtype, plan.n_chan, h, plan.f_ref, plan.t_samp,
-                       [list(r) for r in plan.ranges], int(n_samp)])
+                       [list(r) for r in plan.ranges], int(n_samp), TUNING_VERSION])
 
 
 class Autotuner:

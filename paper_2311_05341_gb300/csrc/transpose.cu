@@ -67,13 +67,15 @@ __global__ void __launch_bounds__(kThreads) transpose_kernel(
   const int32_t c0 = (blockIdx.x % chan_tiles) * (kRowWords * R);
   const int64_t b0 = static_cast<int64_t>(c0) * E;
 
-  // 8 lanes per 128-byte row (rows and strides are 16-byte aligned).
+  // 8 lanes per 128-byte row (rows and strides are 16-byte aligned).  Only
+  // pieces with channels below n_chan: the rows may be columns of wider ones,
+  // and the last of them ends with its memory.
   uint4 v[kLoads];
 #pragma unroll
   for (int k = 0; k < kLoads; ++k) {
     const int i = (tid + k * kThreads) / 8, g = tid % 8;
     v[k] = make_uint4(0u, 0u, 0u, 0u);
-    if (t0 + i < t_end && b0 + 16 * g < in_stride_bytes)
+    if (t0 + i < t_end && b0 + 16 * g < static_cast<int64_t>(n_chan) * E)
       v[k] = __ldcs(reinterpret_cast<const uint4*>(in + (t0 + i) * in_stride_bytes + b0) + g);
   }
 #pragma unroll

@@ -257,7 +257,7 @@ class Plan:
         no ring, the full copies) of every range with a packed copy."""
         import torch
         need = self.input_scratch_bytes(n_samp)
-        if segments > 0 and any(self.info(n_samp)["packed_copy"]):
+        if segments > 0 and self._reads_copies(n_samp):
             try:
                 need = max(need, self.packed_scratch_bytes(n_samp, segments))
             except DDError as err:  # no ring for this plan: the full copies
@@ -267,6 +267,16 @@ class Plan:
         if need == 0:
             return None
         return torch.empty(int(need), dtype=torch.uint8, device=device)
+
+    def _reads_copies(self, n_samp: int) -> bool:
+        """Whether a run with scratch has a range that reads a packed copy.
+        (uint16 ranges on the sum-row tile read the input: scratch for their
+        copies, 1.1 GB in full for 4096 channels x 65536, would stay untouched.)"""
+        info = self.info(n_samp)
+        if self.dtype != "u16":
+            return any(info["packed_copy"])
+        return any(c and (n < 1 or self.run_kernel(r, n)[1])
+                   for r, (c, n) in enumerate(zip(info["packed_copy"], info["n_out"])))
 
     def packed_scratch_bytes(self, n_samp: int, segments: int = 16) -> int:
         """Scratch bytes with which every range with a packed copy runs from

@@ -257,7 +257,7 @@ class Plan:
         no ring, the full copies) of every range with a packed copy."""
         import torch
         need = self.input_scratch_bytes(n_samp)
-        if segments > 0 and self._reads_copies(n_samp):
+        if segments > 0 and self.reads_copies(n_samp):
             try:
                 need = max(need, self.packed_scratch_bytes(n_samp, segments))
             except DDError as err:  # no ring for this plan: the full copies
@@ -268,7 +268,7 @@ class Plan:
             return None
         return torch.empty(int(need), dtype=torch.uint8, device=device)
 
-    def _reads_copies(self, n_samp: int) -> bool:
+    def reads_copies(self, n_samp: int) -> bool:
         """Whether a run with scratch has a range that reads a packed copy.
         (uint16 ranges on the sum-row tile read the input: scratch for their
         copies, 1.1 GB in full for 4096 channels x 65536, would stay untouched.)"""

@@ -541,9 +541,10 @@ void layout_workspace(dd_plan_s* p) {
       rp.off_direct = ws;
       ws += rp.direct.bytes.size();
     }
-    // Sum-row tables: room for both sets, a power of two each, so that the
-    // workspace's size depends on the plan's shape and not on which window
-    // formats its dtype has.
+    // Sum-row tables: two rooms of the power of two that holds the larger set.
+    // The sets of a plan's dtypes (uint16 has one) differ by less, so that its
+    // workspace is as large for each but for the widening slots, unless a set
+    // passes a power of two (8192 channels x 4096 DMs: 11.3 to 12.6 of 16.8 MB).
     if (rp.sums.ok || rp.packed_sums.ok) {
       size_t room = 4096;
       while (room < std::max(rp.sums.bytes.size(), rp.packed_sums.bytes.size())) room *= 2;

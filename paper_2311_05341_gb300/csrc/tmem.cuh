@@ -5,7 +5,8 @@
 // (16-bit sums of high bytes, below 2^16 while the total stays below 2^24) and
 // keeps the low byte: 255 x 256 more fits the lane.  Partial sums so never
 // leave the SM.  A CTA that allocates all 512 columns must be the only one on
-// its SM (its shared memory sees to that).
+// its SM: the 512 threads of 128 registers of both its users (sum-row and
+// direct) take the whole register file.
 #pragma once
 
 #include <cuda_runtime.h>

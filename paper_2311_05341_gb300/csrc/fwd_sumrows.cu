@@ -34,9 +34,14 @@
 // words per thread), so partial sums never leave the SM and every output is
 // stored once.
 //
-// Every mbarrier wait is bounded, and no lane leaves the others in a warp-wide
-// operation (give_up); on timeout the CTA sets kErrTimeout, waits for its
-// copies (drain_copies) and frees its tensor memory.
+// Every mbarrier wait is bounded; a warp that gives one up sets the abort flag,
+// which ends the other waits, and on leaving the CTA sets kErrTimeout, waits for
+// its copies (drain_copies) and frees its tensor memory.  Lanes of a warp may
+// find out one by one, and nothing bounds a warp-wide operation that waits for a
+// lane gone ahead, so warps vote on every wait before they go on or leave: the
+// building warps in build, the adding warps with the byte counts of the copies
+// they issue next (issue_copies).  The votes cost up to 1 % of a launch (8192
+// channels: 70.3, now 70.9 ms through the ring, 78.2 and 78.5 ms from the input).
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -96,18 +101,6 @@ __device__ __forceinline__ bool wait_copies(const Params& p, Ctl* ctl, int g) {
   return tk::mbar_wait(smem_u32(&ctl->raw_full[slot]), (g / kSlots) & 1, p.wait_iters);
 }
 
-// A role gives up: the status word, and the flag that ends the other waits.
-// Lanes of a warp may find out one by one, and nothing bounds a warp-wide
-// operation that waits for a lane gone ahead, so warps vote on every wait
-// before they go on or leave: the building warps in build, the adding warps
-// with the byte counts of the copies they issue next (issue_copies).  The votes
-// cost 0.9 % of a launch from the packed copy (8192 channels: 70.4, now 71.0 ms
-// through the ring), nothing from the input.
-__device__ __forceinline__ void give_up(const Params& p, Ctl* ctl) {
-  atomicOr(p.err, tk::kErrTimeout);
-  ctl->abort = 1;
-}
-
 // After an abort, every role done: the copies still in flight land before the
 // CTA goes on.  The adding warps issue their shares of a group on their own,
 // and one that gave up first leaves its share out; a slot's warps are at most
@@ -115,9 +108,11 @@ __device__ __forceinline__ void give_up(const Params& p, Ctl* ctl) {
 // one have landed).  The arrivals of the warps behind are made here, so that
 // the newest group's phase ends with the bytes that were asked for.
 __device__ __forceinline__ void drain_copies(const Params& p, const Ctl* ctl) {
+#pragma unroll 1
   for (int s = 0; s < kSlots; ++s) {
     int newest = -1;
     uint32_t missing = 0;
+#pragma unroll 1
     for (int w = 0; w < kMainWarps; ++w) {
       int g = ctl->issued_by[w] - 1;              // the warp's newest group ...
       g -= (g % kSlots - s + kSlots) % kSlots;    // ... of this slot
@@ -478,13 +473,13 @@ __device__ __forceinline__ void build_rows(const unsigned char* rec, uint32_t ra
 // 85.7 ms.)
 static_assert(kMaxK <= 4 * kMainWarps, "four channels per adding warp");
 //
-// Also the warp's vote on the wait before it (`ok` of each lane; false where
-// any lane gave up, and then nothing is issued).
-template <int SRC>
+// VOTE: also the warp's vote on the wait before it (`ok` of each lane; false
+// where any lane gave up, and then nothing is issued).
+template <int SRC, bool VOTE>
 __device__ __forceinline__ bool issue_copies(const Params& p, unsigned char* smem, Ctl* ctl,
                                              int64_t w0, int g, const Dir& e, int32_t start,
                                              bool ok = true) {
-  if (g == p.hold_stage) return __all_sync(0xffffffffu, ok);
+  if (g == p.hold_stage) return VOTE ? __all_sync(0xffffffffu, ok) : true;
   constexpr int kBits = format(SRC).bits;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, slot = g % kSlots;
   const uint32_t bar = smem_u32(&ctl->raw_full[slot]);
@@ -497,8 +492,8 @@ __device__ __forceinline__ bool issue_copies(const Params& p, unsigned char* sme
         min(static_cast<int64_t>(row_bytes), (p.stride - at) * kBits / 8));
   constexpr uint32_t kGaveUp = 1u << 24;  // above any sum of bytes, 32 of them below 2^32
   static_assert(format(SRC).raw_bytes < kGaveUp, "byte counts and votes share a word");
-  const uint32_t total = __reduce_add_sync(0xffffffffu, ok ? bytes : kGaveUp);
-  if (total >= kGaveUp) return false;
+  const uint32_t total = __reduce_add_sync(0xffffffffu, VOTE && !ok ? kGaveUp : bytes);
+  if (VOTE && total >= kGaveUp) return false;
   // The slot's last readers were ordinary loads.
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   if (lane == 0) {
@@ -531,10 +526,10 @@ __device__ __forceinline__ void build(const Params& p, unsigned char* smem, Ctl*
   constexpr size_t kRows = row_off(SRC), kRowBytes = static_cast<size_t>(format(SRC).row_words) * 4;
   for (int g = wg; g < n_groups; g += kBuildGroups) {
     const int slot = g % kSlots;
-    const bool ok = wait_copies(p, ctl, g) &&
-                    wait_or_abort(smem_u32(&ctl->rows_empty[slot]), ((g / kSlots) & 1) ^ 1, ctl);
+    const bool ok = wait_or_abort(smem_u32(&ctl->rows_empty[slot]), ((g / kSlots) & 1) ^ 1, ctl) &&
+                    wait_copies(p, ctl, g);
     if (!__all_sync(0xffffffffu, ok)) {
-      if (lane == 0) give_up(p, ctl);
+      ctl->abort = 1;
       return;
     }
     const unsigned char* rec = smem + kRecOff + slot * kRecBytes;
@@ -585,7 +580,7 @@ __device__ __forceinline__ void add_and_store(const Params& p, unsigned char* sm
     for (int g = 0; g < min(kSlots, n_groups); ++g) {
       const int4 v = __ldg(reinterpret_cast<const int4*>(dir + g));
       const Dir e = *reinterpret_cast<const Dir*>(&v);
-      issue_copies<SRC>(p, smem, ctl, w0, g, e, ch < e.k ? __ldg(starts + e.c0 + ch) : 0);
+      issue_copies<SRC, false>(p, smem, ctl, w0, g, e, ch < e.k ? __ldg(starts + e.c0 + ch) : 0);
     }
   }
   for (int g = 0; g < n_groups; ++g) {
@@ -597,16 +592,14 @@ __device__ __forceinline__ void add_and_store(const Params& p, unsigned char* sm
       const uint4 v = *reinterpret_cast<const uint4*>(offs + kNextDir);
       const Dir e = *reinterpret_cast<const Dir*>(&v);
       const int ch = min(w + kMainWarps * lane, kMaxK - 1);
-      ok = issue_copies<SRC>(p, smem, ctl, w0, g + kSlots, e,
-                             static_cast<int32_t>(offs[kNextStart + ch]), ok);
+      ok = issue_copies<SRC, true>(p, smem, ctl, w0, g + kSlots, e,
+                                   static_cast<int32_t>(offs[kNextStart + ch]), ok);
     } else {
       ok = __all_sync(0xffffffffu, ok);
     }
     if (!ok) {
-      if (lane == 0) {
-        ctl->issued_by[w] = min(g + kSlots, n_groups);
-        give_up(p, ctl);
-      }
+      ctl->issued_by[w] = min(g + kSlots, n_groups);
+      ctl->abort = 1;
       return;
     }
 #pragma unroll
@@ -714,7 +707,10 @@ __global__ void __launch_bounds__(kThreads, 1) sum_row_kernel(const __grid_const
   }
   if constexpr (LANES16) tmem::fence_before();
   __syncthreads();
-  if (ctl->abort && threadIdx.x == 0) drain_copies(p, ctl);
+  if (ctl->abort && threadIdx.x == 0) {
+    atomicOr(p.err, tk::kErrTimeout);
+    drain_copies(p, ctl);
+  }
   if constexpr (LANES16) {
     tmem::fence_after();
     __syncwarp();
@@ -754,7 +750,10 @@ __global__ void __launch_bounds__(kThreads, 1) sum_row_batch_kernel(const BatchA
     const bool aborted = !fresh && ctl->abort;
     if (threadIdx.x == 0) {
       if (!fresh) {
-        if (aborted) drain_copies(bc->p, ctl);
+        if (aborted) {
+          atomicOr(bc->p.err, tk::kErrTimeout);
+          drain_copies(bc->p, ctl);
+        }
         for (int s = 0; s < kSlots; ++s) {
           mbar_inval(smem_u32(&ctl->raw_full[s]));
           mbar_inval(smem_u32(&ctl->rows_full[s]));

@@ -471,10 +471,9 @@ __device__ __forceinline__ void build_rows(const unsigned char* rec, uint32_t ra
 // the packed copy: 67.7 ms; one building warp per warpgroup issuing all of
 // them 68.0 ms, half by each 73.1 ms; from the input itself 78.3, 85.3 and
 // 85.7 ms.)
-static_assert(kMaxK <= 4 * kMainWarps, "four channels per adding warp");
-//
 // VOTE: also the warp's vote on the wait before it (`ok` of each lane; false
 // where any lane gave up, and then nothing is issued).
+static_assert(kMaxK <= 4 * kMainWarps, "four channels per adding warp");
 template <int SRC, bool VOTE>
 __device__ __forceinline__ bool issue_copies(const Params& p, unsigned char* smem, Ctl* ctl,
                                              int64_t w0, int g, const Dir& e, int32_t start,

@@ -326,9 +326,17 @@ void add_pattern_units(const RangePlan& rp, int32_t n_chan, bool nibbles, int ki
 bool sum_rows_faster(const SumTables& t, const RangePlan& rp, int32_t n_chan, bool nibbles,
                      int kind, int64_t outputs, bool overlapped) {
   std::vector<UnitCost> sums, pattern;
-  sums.reserve(t.unit_cycles.size());
-  add_sum_row_units(t, false, outputs, &sums);
   add_pattern_units(rp, n_chan, nibbles, kind, outputs, &pattern);
+  // From 64 waves on the last one does not tell (and a plan may have millions
+  // of blocks): their mean cost.
+  const int64_t halves = sum_row_halves(t.src, 0, outputs);
+  const int64_t blocks = static_cast<int64_t>(t.unit_cycles.size());
+  if (blocks * halves >= 64 * tk::kSms) {
+    sums.push_back({t.unit_total / static_cast<double>(blocks), blocks * halves});
+  } else {
+    sums.reserve(t.unit_cycles.size());
+    add_sum_row_units(t, false, outputs, &sums);
+  }
   return launch_cycles(sums, overlapped) < launch_cycles(pattern, overlapped);
 }
 
@@ -400,6 +408,7 @@ void build_sum_tables(const RangePlan& rp, int32_t n_chan, int64_t max_sample, i
   out->off_dir = static_cast<int32_t>(off_dir);
   out->off_start = static_cast<int32_t>(off_start);
   for (const Block& b : blocks) {
+    out->unit_total += b.unit;
     out->unit_cycles.push_back(b.unit);
     out->batch_cycles.push_back(b.batch_unit);
   }

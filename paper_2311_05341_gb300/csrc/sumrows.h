@@ -195,6 +195,7 @@ struct SumTables {
   // and in the persistent kernel.
   std::vector<double> unit_cycles;
   std::vector<double> batch_cycles;
+  double unit_total = 0.0;  // of unit_cycles
   std::vector<unsigned char> bytes;
 };
 

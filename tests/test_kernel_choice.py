@@ -100,3 +100,11 @@ def test_packed_uint16_never_reads_the_input_with_its_copys_tables():
     plan = _plan("u16", 150, 130, 0.4)
     plan.set_tile(0, "packed")
     assert plan.run_kernel(0, 30000) == ("sum-rows", False)
+
+
+def test_choice_over_many_waves():
+    """Past 64 waves the mean of the units decides, as it nearly does just below."""
+    plan = _plan("u8", 600, 1000, 0.2)
+    per_wave = 152 * 736 // 8  # 8 blocks of 128 DMs
+    for waves in (50, 63, 64, 65, 2000):
+        assert plan.run_kernel(0, waves * per_wave, scratch=False)[0] == "sum-rows"

@@ -19,9 +19,9 @@
 // span.  The planner picks K per group to make the whole cheapest: 5300 words
 // per channel at 8192 channels and 4096 trials (K = 15, 17 rows, 21 moves on
 // average), where the pattern tile moves 12000.  Measured there (262144
-// uint8 samples, one launch): 67.8 ms from the packed copy (pattern tile 153.5)
-// and 78.3 ms from the input (170.0); uint16, 4096 channels x 65536, 3072
-// trials 19.1 ms (29.6).  Per group the adders take 3300 cycles, of which 2400
+// uint8 samples, one launch): 68.4 ms from the packed copy (pattern tile 153.5)
+// and 78.5 ms from the input (170.0); uint16, 4096 channels x 65536, 3072
+// trials 19.3 ms (29.6).  Per group the adders take 3300 cycles, of which 2400
 // are adds against 1472 of the bare reads, 500 the copies' issue and 300 the
 // lanes' high bytes; the builders are as long.  One building warpgroup with
 // two buffers and groups of 22 channels ran 90 ms: a warp's chain of moves
@@ -468,7 +468,7 @@ __device__ __forceinline__ void build_rows(const unsigned char* rec, uint32_t ra
 // g % kSlots, by adding warp w: lane i < 4 the window of channel w + 8 i, warp
 // 0 the record too.  A bulk copy takes its warp about 130 cycles whatever its
 // size, so the copies are spread over the adding warps.  (8192 channels, from
-// the packed copy: 67.7 ms; one building warp per warpgroup issuing all of
+// the packed copy, before the votes: 67.7 ms; one building warp per warpgroup issuing all of
 // them 68.0 ms, half by each 73.1 ms; from the input itself 78.3, 85.3 and
 // 85.7 ms.)
 // VOTE: also the warp's vote on the wait before it (`ok` of each lane; false

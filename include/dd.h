@@ -545,13 +545,15 @@ dd_status dd_run_u8_noalloc_status(void* stream);
 /* ---------------------------------------------------------------------------
  * Persistent batches: many beams (plans of different channel counts, dtypes,
  * sampling times and DM plans) dedispersed by persistent launches of the
- * tiled kernels -- one for the ranges on the pattern tile, one for those on
+ * tiled kernels -- one for the ranges on each variant of the pattern tile, one
+ * for each window format of the sum-row tile (which takes the pattern tile's
+ * place where its units, over the whole batch, end sooner), one for those on
  * offset tiles -- whose CTAs take (beam range, DM block, time tile) work items
  * from a device counter, longest items first.  The paper tunes its tile
  * parameters per telescope and plan (Sec. 4.1); here each plan's tile is
  * chosen before the batch is built (dd_plan_set_tile), so the batch mixes
- * tiles.  The batch keeps pointers to its plans, which must outlive it and
- * stay uploaded.  Device memory is the caller's (dd_batch_workspace_bytes).
+ * tiles.  The batch keeps pointers to its plans, which must outlive it, keep
+ * their tiles and stay uploaded.  Device memory is the caller's (dd_batch_workspace_bytes).
  * ------------------------------------------------------------------------- */
 typedef struct dd_batch_s* dd_batch;
 
@@ -568,9 +570,9 @@ dd_status dd_batch_destroy(dd_batch batch);
 dd_status dd_batch_workspace_bytes(dd_batch batch, size_t* bytes);
 /* Number of work items and jobs (plan ranges) of the batch. */
 dd_status dd_batch_info(dd_batch batch, int64_t* n_items, int32_t* n_jobs);
-/* Kernel launches one dd_batch_run makes (one per pattern-tile variant present,
- * one if any range is on an offset tile, and one packing launch per plan with
- * a DD_TILE_PACKED range). */
+/* Kernel launches one dd_batch_run makes (one per pattern-tile variant and
+ * sum-row format present, one if any range is on an offset tile, and one packing
+ * launch per packed copy that a range reads). */
 dd_status dd_batch_launches(dd_batch batch, int32_t* n_launches);
 /* Copy the work list into caller device memory (256-byte aligned, >= the
  * workspace bytes) and bind it; synchronises `stream`. */
@@ -592,7 +594,8 @@ dd_status dd_batch_plan_scratch_bytes(dd_batch batch, int32_t plan, size_t* byte
  * first writes the packed copies (one packing launch per such plan), and the
  * persistent launches read them.  The scratch is in use while runs are.
  * Errors: as dd_batch_bind; DD_ERR_UNSUPPORTED for missing scratch,
- * DD_ERR_BUDGET for too little, DD_ERR_SHAPE for a misaligned one. */
+ * DD_ERR_BUDGET for too little, DD_ERR_SHAPE for a misaligned one,
+ * DD_ERR_INVALID_ARG for a plan that left the sum-row tile since. */
 dd_status dd_batch_bind_scratch(dd_batch batch, const void* const* d_in,
                                 const int64_t* in_row_stride, void* const* d_out,
                                 void* const* d_scratch, const size_t* scratch_bytes,

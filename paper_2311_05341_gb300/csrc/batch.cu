@@ -452,6 +452,10 @@ dd_status dd_batch_bind_scratch(dd_batch batch, const void* const* d_in,
       return fail(DD_ERR_SHAPE, "batch input/output alignment or stride");
     const RangePlan& rp = p->ranges[jr.range];
     const SumTables* sums = jr.sums ? batch->sums_of(rp) : nullptr;
+    if (jr.sums && !sums)  // its items are the sum-row tile's
+      return fail(DD_ERR_INVALID_ARG, "batch plan " + std::to_string(jr.plan) + " range " +
+                                          std::to_string(jr.range) +
+                                          " left the tile the batch was built for");
     if (rp.tile_ok && (sums ? sums->src == sr::kPairs
                             : tk::packed_copy_kind(rp.tile_kind))) {  // reads its packed copy
       std::vector<int32_t> range_copy;

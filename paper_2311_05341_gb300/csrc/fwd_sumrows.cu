@@ -468,9 +468,9 @@ __device__ __forceinline__ void build_rows(const unsigned char* rec, uint32_t ra
 // g % kSlots, by adding warp w: lane i < 4 the window of channel w + 8 i, warp
 // 0 the record too.  A bulk copy takes its warp about 130 cycles whatever its
 // size, so the copies are spread over the adding warps.  (8192 channels, from
-// the packed copy, before the votes: 67.7 ms; one building warp per warpgroup issuing all of
-// them 68.0 ms, half by each 73.1 ms; from the input itself 78.3, 85.3 and
-// 85.7 ms.)
+// the packed copy, before the votes: 67.7 ms; one building warp per warpgroup
+// issuing all of them 68.0 ms, half by each 73.1 ms; from the input itself 78.3,
+// 85.3 and 85.7 ms.)
 // VOTE: also the warp's vote on the wait before it (`ok` of each lane; false
 // where any lane gave up, and then nothing is issued).
 static_assert(kMaxK <= 4 * kMainWarps, "four channels per adding warp");

@@ -130,8 +130,8 @@ void choose_sums(dd_batch_s* b) {
       if (!t || n_out <= 0) continue;
       ++jobs[t->src];
       add_sum_row_units(*t, true, n_out, &sums[t->src]);
-      add_pattern_units(rp, b->plans[i]->n_chan, b->plans[i]->dtype == DD_U4, rp.tile_kind, n_out,
-                        &pattern[t->src]);
+      pattern[t->src].push_back(pattern_units(rp, b->plans[i]->n_chan,
+                                              b->plans[i]->dtype == DD_U4, rp.tile_kind, n_out));
     }
   constexpr double kFavour = 0.95;
   auto cheaper = [](const UnitCost& a, const UnitCost& c) { return a.cycles < c.cycles; };

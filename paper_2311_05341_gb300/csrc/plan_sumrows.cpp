@@ -269,10 +269,15 @@ bool build_block(const RangePlan& rp, int32_t n_chan, int lane_chans, const Form
 
 }  // namespace
 
-double launch_cycles(const std::vector<UnitCost>& sorted, bool overlapped) {
+namespace {
+
+// launch_cycles of unit(0) .. unit(n_costs - 1).
+template <typename Unit>
+double launch_cycles_of(int64_t n_costs, Unit unit, bool overlapped) {
   int64_t n = 0;
   double total = 0;
-  for (const UnitCost& u : sorted) {
+  for (int64_t i = 0; i < n_costs; ++i) {
+    const UnitCost u = unit(i);
     n += u.count;
     total += u.cycles * static_cast<double>(u.count);
   }
@@ -280,17 +285,24 @@ double launch_cycles(const std::vector<UnitCost>& sorted, bool overlapped) {
   if (overlapped)
     return std::max(static_cast<double>(n) / tk::kSms, 0.5) * total / static_cast<double>(n);
   const int64_t waves = (n + tk::kSms - 1) / tk::kSms;
-  if (waves == 1) return sorted.back().cycles;
+  if (waves == 1) return unit(n_costs - 1).cycles;
   // The share of the units (by cost) that frees the SMs of the last wave.
   const double share = static_cast<double>(n - (waves - 1) * tk::kSms) / tk::kSms;
   double start = 0, seen = 0;
-  for (const UnitCost& u : sorted) {
+  for (int64_t i = 0; i < n_costs && seen < share * static_cast<double>(n); ++i) {
+    const UnitCost u = unit(i);
     start = u.cycles;
     seen += static_cast<double>(u.count);
-    if (seen >= share * static_cast<double>(n)) break;
   }
   return static_cast<double>(waves - 2) * total / static_cast<double>(n) + start +
-         sorted.back().cycles;
+         unit(n_costs - 1).cycles;
+}
+
+}  // namespace
+
+double launch_cycles(const std::vector<UnitCost>& sorted, bool overlapped) {
+  return launch_cycles_of(
+      static_cast<int64_t>(sorted.size()), [&](int64_t i) { return sorted[i]; }, overlapped);
 }
 
 void add_sum_row_units(const SumTables& t, bool batch, int64_t outputs,
@@ -299,8 +311,8 @@ void add_sum_row_units(const SumTables& t, bool batch, int64_t outputs,
   for (double c : batch ? t.batch_cycles : t.unit_cycles) units->push_back({c, halves});
 }
 
-void add_pattern_units(const RangePlan& rp, int32_t n_chan, bool nibbles, int kind,
-                       int64_t outputs, std::vector<UnitCost>* units) {
+UnitCost pattern_units(const RangePlan& rp, int32_t n_chan, bool nibbles, int kind,
+                       int64_t outputs) {
   // Cycles of a 64-DM unit, per channel and besides, as measured: one kind and
   // bin each (7 % around them).
   struct {
@@ -320,24 +332,23 @@ void add_pattern_units(const RangePlan& rp, int32_t n_chan, bool nibbles, int ki
            31000};
   }
   const int ts = tk::pat_tile_samples(kind, rp.tile_h);
-  units->push_back({c.fixed + c.per_chan * n_chan, (outputs + ts - 1) / ts * rp.tile_n_blocks});
+  return {c.fixed + c.per_chan * n_chan, (outputs + ts - 1) / ts * rp.tile_n_blocks};
 }
 
 bool sum_rows_faster(const SumTables& t, const RangePlan& rp, int32_t n_chan, bool nibbles,
                      int kind, int64_t outputs, bool overlapped) {
-  std::vector<UnitCost> sums, pattern;
-  add_pattern_units(rp, n_chan, nibbles, kind, outputs, &pattern);
-  // From 64 waves on the last one does not tell (and a plan may have millions
-  // of blocks): their mean cost.
+  const UnitCost pattern = pattern_units(rp, n_chan, nibbles, kind, outputs);
   const int64_t halves = sum_row_halves(t.src, 0, outputs);
   const int64_t blocks = static_cast<int64_t>(t.unit_cycles.size());
-  if (blocks * halves >= 64 * tk::kSms) {
-    sums.push_back({t.unit_total / static_cast<double>(blocks), blocks * halves});
-  } else {
-    sums.reserve(t.unit_cycles.size());
-    add_sum_row_units(t, false, outputs, &sums);
-  }
-  return launch_cycles(sums, overlapped) < launch_cycles(pattern, overlapped);
+  // From 64 waves on the last one does not tell (and a plan may have millions
+  // of blocks): their mean cost.
+  const UnitCost mean{t.unit_total / static_cast<double>(blocks), blocks * halves};
+  const double sums =
+      mean.count >= 64 * tk::kSms
+          ? launch_cycles_of(1, [&](int64_t) { return mean; }, overlapped)
+          : launch_cycles_of(
+                blocks, [&](int64_t i) { return UnitCost{t.unit_cycles[i], halves}; }, overlapped);
+  return sums < launch_cycles_of(1, [&](int64_t) { return pattern; }, overlapped);
 }
 
 void build_sum_tables(const RangePlan& rp, int32_t n_chan, int64_t max_sample, int src,

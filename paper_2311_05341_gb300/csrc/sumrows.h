@@ -210,12 +210,12 @@ struct UnitCost {
   int64_t count;
 };
 double launch_cycles(const std::vector<UnitCost>& sorted, bool overlapped);
-// The units of `outputs` outputs of a range on the sum-row tile, and on the
-// pattern kernel `kind` (its tables' kind or the packed copy's), appended.
+// The units of `outputs` outputs of a range on the sum-row tile, appended, and on
+// the pattern kernel `kind` (its tables' kind or the packed copy's).
 void add_sum_row_units(const SumTables& t, bool batch, int64_t outputs,
                        std::vector<UnitCost>* units);
-void add_pattern_units(const RangePlan& rp, int32_t n_chan, bool nibbles, int kind,
-                       int64_t outputs, std::vector<UnitCost>* units);
+UnitCost pattern_units(const RangePlan& rp, int32_t n_chan, bool nibbles, int kind,
+                       int64_t outputs);
 // Whether the sum-row tile takes the launch.  Its 128-DM units leave more of
 // the chip idle than the pattern tile's 64-DM ones where there are few: 150
 // channels x 130 DMs x 60000 uint8 outputs make 164 units, 2 waves of 66 us

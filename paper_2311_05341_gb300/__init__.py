@@ -12,7 +12,6 @@ direct transform of Eq. 3 (Sec. 2 of the paper); see include/dd.h.
 """
 from __future__ import annotations
 
-import contextlib
 import ctypes
 
 import numpy as np
@@ -44,6 +43,19 @@ def build(force: bool = False) -> str:
 _PADDING_ALONE = 56 << 20
 
 
+def _rows_for(x_tm, shape, n_samp: int, whole: bool):
+    """The output that transpose makes: zero wherever it writes nothing (whole:
+    it writes every sample)."""
+    import torch
+    if not whole or (shape[1] > n_samp and
+                     shape[0] * shape[1] * x_tm.element_size() < _PADDING_ALONE):
+        return torch.zeros(shape, dtype=x_tm.dtype, device=x_tm.device)
+    out = torch.empty(shape, dtype=x_tm.dtype, device=x_tm.device)
+    if shape[1] > n_samp:
+        out[:, n_samp:] = 0
+    return out
+
+
 def transpose(x_tm, n_chan: int | None = None, out=None, t_begin: int = 0,
               t_end: int | None = None, stream=None):
     """Time-major cuda tensor x_tm [n_samp][stride >= n_chan] -> channel-major
@@ -56,16 +68,12 @@ def transpose(x_tm, n_chan: int | None = None, out=None, t_begin: int = 0,
     if out is None:
         per = 16 // x_tm.element_size()
         shape = (nc, (n_samp + per - 1) // per * per)
-        with contextlib.nullcontext() if stream is None else torch.cuda.stream(stream):
-            if (t_begin == 0 and (t_end is None or int(t_end) == n_samp)
-                    and (shape[1] == n_samp or
-                         nc * shape[1] * x_tm.element_size() >= _PADDING_ALONE)):
-                # Every sample is written; only the rows' padding is zeroed.
-                out = torch.empty(shape, dtype=x_tm.dtype, device=x_tm.device)
-                if shape[1] > n_samp:
-                    out[:, n_samp:] = 0
-            else:
-                out = torch.zeros(shape, dtype=x_tm.dtype, device=x_tm.device)
+        whole = t_begin == 0 and (t_end is None or int(t_end) == n_samp)
+        if stream is None:
+            out = _rows_for(x_tm, shape, n_samp, whole)
+        else:
+            with torch.cuda.stream(stream):
+                out = _rows_for(x_tm, shape, n_samp, whole)
     te = n_samp if t_end is None else int(t_end)
     check(_lib.load().dd_transpose(DTYPES[dt], x_tm.data_ptr(), x_tm.stride(0), nc,
                                    out.data_ptr(), out.stride(0), int(t_begin), te,

@@ -114,8 +114,8 @@ const dd::SumTables* batch_sums(const dd::RangePlan& rp) {
 // (sum_rows_faster) on the units of all ranges of the format, which one
 // persistent launch takes; overlapped with the batch's other launches, if any.
 // Measured on 1134 batches of 1 and 4 equal beams (150 to 2000 channels, 64 to
-// 1000 DMs, 0.3 to 2 samples a step, every format): 1.25 times the pattern
-// tile's speed on average and nine at 0.93 to 0.98 of it (on sum rows always:
+// 1000 DMs, 0.3 to 2 samples a step, every format): 1.26 times the pattern
+// tile's speed on average and eight at 0.94 to 0.98 of it (on sum rows always:
 // 52, down to 0.75).  The 5 % in favour of the sum rows are within what the
 // costs are good for.
 void choose_sums(dd_batch_s* b) {
